@@ -102,7 +102,9 @@ typedef struct brs_params {
  * Box blocks (BRS_BOX): bx, by, bz must divide nx, ny, nz (BRS_ERR_ARG otherwise; one
  * inverse then serves every box, Sec. 4.3).  BRS_PLANE_AUTO selects FP64 CUDA-core math
  * for BRS_F64 and, for BRS_F32, split-TF32 tensor cores when bx*by*bz is a multiple of 4
- * and >= 32, else FP32 CUDA cores.
+ * and > 64 (> 32 for chaotic GS), or >= 32 with a side over 16, else FP32 CUDA cores.
+ * CUDA-core boxes with sides of at most 16 are solved in the box's sine basis, in one pass
+ * over the grid per sweep (per colour for GS) and without right-hand-side storage.
  * y-line and z-line blocks (BRS_YLINE, BRS_ZLINE): the full-extent lines along y or z,
  * solved exactly.  A y-line (z-line) sweep is the x-line sweep of the grid with its axes
  * permuted to (y, x, z) ((z, x, y)) and the coefficients permuted with them, so the

@@ -61,6 +61,7 @@ struct BoxState {
     void* Rf = nullptr;
     void* ftab = nullptr; // [3][n] int2: the fold's passes (x, y, z), the last into class order
     void* utab = nullptr; // [3][n] int2: the unfold's passes (z, y, x), the first from class order
+    void* sine = nullptr; // one-pass form in the box's sine basis (box_sine.cu); null otherwise
 };
 
 BoxState* bs(brs_ctx* c) { return static_cast<BoxState*>(c->box); }
@@ -618,6 +619,8 @@ int box_pass(brs_ctx* c, const T* uin, T* uout, const T* b, const long long* row
     const brs_params& p = c->p;
     if (M == 0)
         return BRS_OK;
+    if (B->sine)
+        return box_sine_pass(B->sine, p.dtype, uin, uout, b, rows, M, s);
     cudaError_t e = cudaSuccess;
     if (B->split == 0 && B->fold)
         return box_pass_fold<T>(c, uin, uout, b, rows, M, s);
@@ -790,6 +793,25 @@ int box_setup(brs_ctx* c)
         // K-major rows of n FP32 must be 16-byte multiples and span one 32-value TMA box
         return BRS_ERR_UNSUPPORTED;
     }
+    // Boxes with sides of at most 16: one fused pass in the box's sine basis (box_sine.cu), in the
+    // context dtype.  FP32 contexts that the automatic choice puts on the tensor cores keep the
+    // split-TF32 product where its values differ visibly: its accumulators truncate, and after 20
+    // sweeps the iterates are 2e-5 (2-norm) from the FP32 solve's at 128 cells under Jacobi and at
+    // 64 under Gauss-Seidel, growing with the cells (9e-6 and 1.5e-5 at half that; the FP32 solve
+    // itself is within 2e-6 of FP64).  Named tensor arithmetic is kept too.
+    // BRSMOOTH_BOX_SINE=0, or a choice among the dense forms (BRSMOOTH_BOX_FOLD), keeps the
+    // dense inverse.  256^3, us per Jacobi / Gauss-Seidel sweep, dense -> sine, same box: FP64
+    // 8^3 2724 / 3921 -> 862 / 868, 4^3 1936 / 2023 -> 532 / 537, 2^3 1159 / 1170 -> 357 / 361;
+    // FP32 CUDA cores 8^3 412 / 490 -> 52 / 75, 2^3 310 / 328 -> 80 / 91; 64^3 FP64 8^3 576 /
+    // 1149 -> 19 / 23.
+    const bool tensor = math == BRS_PLANE_TF32 || math == BRS_PLANE_3XTF32;
+    const bool near = p.plane_math == BRS_PLANE_AUTO &&
+                      n * (p.method == BRS_CHAOTIC_GS ? 2 : 1) <= 64;
+    const bool sine = (!tensor || near) && box_sine_takes(p) &&
+                      env_int("BRSMOOTH_BOX_SINE", 1) != 0 &&
+                      std::getenv("BRSMOOTH_BOX_FOLD") == nullptr;
+    if (sine)
+        math = BRS_PLANE_SIMT;
     B->math = math;
     B->split = math == BRS_PLANE_3XTF32 ? 3 : math == BRS_PLANE_TF32 ? 1 : 0;
     B->bn = n >= 128 ? 128 : n >= 64 ? 64 : 32;
@@ -799,9 +821,12 @@ int box_setup(brs_ctx* c)
     if (e != cudaSuccess)
         return brs_cuda_status(e);
     // the inverse, once (Sec. 4.3)
-    const std::vector<double> inv = block_inverse(p.bx, p.by, p.bz, p.ax, p.ay, p.az);
+    const std::vector<double> inv =
+        sine ? std::vector<double>() : block_inverse(p.bx, p.by, p.bz, p.ax, p.ay, p.az);
     int rc = BRS_OK;
-    if (B->split) {
+    if (sine) {
+        rc = box_sine_setup(p, c->omega, &B->sine);
+    } else if (B->split) {
         rc = brs_tc::upload_split(&B->inv, &B->inv_lo, inv);
     } else if (p.dtype == BRS_F64) {
         rc = upload(&B->inv, inv);
@@ -831,6 +856,8 @@ int box_setup(brs_ctx* c)
         }
     }
     rc = upload(reinterpret_cast<void**>(&B->rows), rows);
+    if (sine)
+        return rc;  // no right-hand-side rows, no dense operands
     std::vector<int> off(n);
     for (int l = 0; l < n; ++l) {
         const int lx = l % p.bx, ly = (l / p.bx) % p.by, lz = l / (p.bx * p.by);
@@ -888,6 +915,7 @@ void box_teardown(brs_ctx* c)
     for (void* q : bufs)
         if (q)
             cudaFree(q);
+    box_sine_teardown(B->sine);
     delete B;
     c->box = nullptr;
 }
