@@ -113,11 +113,13 @@ typedef struct brs_params {
  * runs all its sweeps, and permutes u back: three grid passes per call, whatever nsweeps.
  * Chaotic GS visits the lines in the permuted order.  Limits: the line length (ny or nz)
  * as for x-lines, and nz <= 65535 (y-lines) or ny <= 65535 (z-lines).
- * FP64 x-line blocks: the sweeps run on line-major copies of u and b (cell index i
- * outermost, the lines of each row k split by colour (j+k) mod 2), so the context holds
- * three more buffers of nx*nz*2*ceil(ny/2) doubles and each brsmooth_sweep call copies u
- * and b in and u back (three grid passes per call).  Each line is eliminated from both ends
- * by two threads with pivots factored once (Sec. 2 / Sec. 4.3: invert once, reuse).
+ * FP64 x-line blocks: each line is eliminated from both ends by two threads with pivots
+ * factored once (Sec. 2 / Sec. 4.3: invert once, reuse), on the caller's arrays (the context
+ * holds one grid-sized buffer for b scaled by the pivots).  Grids of many lines (at least 320
+ * per SM) also hold three buffers of nx*nz*2*ceil(ny/2) doubles: calls of 4 or more sweeps run
+ * on line-major copies there (cell index i outermost, the lines of each row k split by colour
+ * (j+k) mod 2), u and b copied in and u back per call (three grid passes).  Both forms do the
+ * same operations in the same order: the iterates are the same bit for bit.
  * Chaotic GS on these contexts visits the lines in two colours, j+k even then odd, each
  * colour reading the other colour's newest values: the red-black line order, one
  * admissible order of the chaotic scheme, deterministic.  BRSMOOTH_LINE_SEQ=0 in the

@@ -19,6 +19,7 @@
 
 #include "brs_internal.cuh"
 #include "line_impl.cuh"
+#include "line_tile.cuh"
 
 namespace {
 
@@ -582,6 +583,7 @@ extern "C" int brsmooth_adjoint_sweep(brs_ctx* c, void* lam, const void* u_k, co
         cudaFree(A->xctx->scratch);
         A->xctx->scratch = nullptr;
         line_seq_teardown(A->xctx);
+        line_tile_teardown(A->xctx);
         A->xstatus = A->xctx->dev_status;
         A->xctx->dev_status = c->dev_status;
     }

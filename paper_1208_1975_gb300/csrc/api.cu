@@ -12,6 +12,7 @@
 #include "brs_internal.cuh"
 #include "batched.cuh"
 #include "box.cuh"
+#include "line_tile.cuh"
 #include "plane.cuh"
 
 namespace {
@@ -173,6 +174,7 @@ void free_ctx(brs_ctx* c)
         return;
     line_teardown(c);
     line_seq_teardown(c);
+    line_tile_teardown(c);
     plane_teardown(c);
     box_teardown(c);
     batched_teardown(c);
@@ -289,10 +291,15 @@ int brsmooth_create(const brs_params* p, brs_ctx** out)
     *c->dev_status = 0;
     if (p->block == BRS_XLINE) {
         rc = line_setup(c);
-        // FP64 lines: the twisted-elimination path (BRSMOOTH_LINE_SEQ=0: the lane-scan kernel)
+        // FP64 lines: the elimination from both ends (BRSMOOTH_LINE_SEQ=0: the lane-scan
+        // kernel), on the caller's layout; grids with enough lines also hold the line-major
+        // form for calls of several sweeps
         const char* ev = std::getenv("BRSMOOTH_LINE_SEQ");
-        if (rc == BRS_OK && p->dtype == BRS_F64 && !(ev && ev[0] == '0'))
-            rc = line_seq_setup(c);
+        if (rc == BRS_OK && p->dtype == BRS_F64 && !(ev && ev[0] == '0')) {
+            rc = line_tile_setup(c);
+            if (rc == BRS_OK && line_seq_takes(c))
+                rc = line_seq_setup(c);
+        }
     } else if (p->block == BRS_XYPLANE)
         rc = plane_setup(c);
     else if (p->block == BRS_BOX)
@@ -345,8 +352,10 @@ int brsmooth_sweep(brs_ctx* c, void* u, const void* b, int nsweeps, void* stream
         return batched_sweep(c, u, b, nsweeps, s);
     if (c->perm)
         return perm_sweep(c, u, b, nsweeps, s);
-    if (c->lseq)
+    if (c->lseq && nsweeps >= kLineSeqMinSweeps)
         return line_seq_sweep(c, u, b, nsweeps, s);
+    if (c->ltile)
+        return line_tile_sweep(c, u, b, nsweeps, s);
     if (c->plane) {
         // several plane sweeps in one call: the x-sine form, where the context has it
         rc = plane_modes_sweep(c, u, b, nsweeps, s);

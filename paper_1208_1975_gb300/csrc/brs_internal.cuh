@@ -83,6 +83,8 @@ struct brs_ctx {
     void* adjoint = nullptr;
     // FP64 x-line sweeps on the line-major copy (owned by line_seq.cu); null otherwise
     void* lseq = nullptr;
+    // FP64 x-line sweeps on the caller's layout (owned by line_tile.cu); null otherwise
+    void* ltile = nullptr;
     // y-line / z-line blocks (api.cu): an x-line context of the permuted grid and the
     // permuted copies of u and b it sweeps
     brs_ctx* perm = nullptr;
@@ -102,6 +104,12 @@ int line_sweep_launch(brs_ctx* c, const void* uin, void* uout, const void* b, cu
 
 // FP64 x-line path (line_seq.cu): one thread per half line, elimination from both ends,
 // on a line-major colour-split copy of u and b made by each call.
+// Taken for grids of at least 20 16-line tasks per SM in calls of at least 4 sweeps, where the
+// three copies per call are paid back (us per sweep in calls of 1 / 3 / 8 / 30, line-major
+// against line_tile.cu, same box: 256^3 Jacobi 400 / 279 / 240 / 223 against 325 / 293 / 255 /
+// 250; 192^3, 15 tasks per SM, 185 / 130 / 112 / 105 against 151 / 135 / 107 / 105).
+constexpr int kLineSeqMinSweeps = 4;
+bool line_seq_takes(const brs_ctx* c);
 int line_seq_setup(brs_ctx* c);
 void line_seq_teardown(brs_ctx* c);
 int line_seq_sweep(brs_ctx* c, void* u, const void* b, int nsweeps, cudaStream_t s);

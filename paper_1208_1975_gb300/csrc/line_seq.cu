@@ -393,6 +393,14 @@ int pick_shape(brs_ctx* c, long long tasks, bool persist, Shape* sh)
 
 }  // namespace
 
+bool line_seq_takes(const brs_ctx* c)
+{
+    int sms = 0;
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
+    const int force = env_int("BRSMOOTH_LINE_SEQ", 1);  // 2: every grid (measurements, tests)
+    return force == 2 || (long long)c->p.ny * c->p.nz >= 20ll * kLinesPerWarp * sms;
+}
+
 int line_seq_setup(brs_ctx* c)
 {
     const brs_params& p = c->p;
