@@ -116,7 +116,7 @@ typedef struct brs_params {
  * FP64 x-line blocks: each line is eliminated from both ends by two threads with pivots
  * factored once (Sec. 2 / Sec. 4.3: invert once, reuse), on the caller's arrays (the context
  * holds one grid-sized buffer for b scaled by the pivots).  Grids of many lines (at least 320
- * per SM) also hold three buffers of nx*nz*2*ceil(ny/2) doubles: calls of 4 or more sweeps run
+ * per SM) hold three buffers of nx*nz*2*ceil(ny/2) doubles instead: calls of 4 or more sweeps run
  * on line-major copies there (cell index i outermost, the lines of each row k split by colour
  * (j+k) mod 2), u and b copied in and u back per call (three grid passes).  Both forms do the
  * same operations in the same order: the iterates are the same bit for bit.

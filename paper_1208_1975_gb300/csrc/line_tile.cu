@@ -328,7 +328,8 @@ int line_tile_setup(brs_ctx* c)
     cudaError_t e = cudaMalloc(&S->tab, tab.size() * sizeof(double));
     if (e == cudaSuccess)
         e = cudaMemcpy(S->tab, tab.data(), tab.size() * sizeof(double), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess)
+    // calls of 4 or more sweeps scale b into bs, unless the line-major form takes them
+    if (e == cudaSuccess && !line_seq_takes(c))
         e = cudaMalloc(&S->bs, (size_t)c->cells * sizeof(double));
     a.tab = S->tab;
     const size_t smem = tile_smem(a, kLines);
@@ -377,7 +378,7 @@ int line_tile_sweep(brs_ctx* c, void* u, const void* b, int nsweeps, cudaStream_
     int mode = B_PLAIN, rc = BRS_OK;
     // b scaled once where that pays: 24 bytes per cell and a launch (2 us) against one FP64
     // operation per cell and sweep (626 G/s).  The results are the same bit for bit.
-    if (nsweeps >= 4 && (double)(nsweeps - 4) * c->cells > 1.25e6) {
+    if (S->bs && nsweeps >= 4 && (double)(nsweeps - 4) * c->cells > 1.25e6) {
         const long long need = (c->cells + 255) / 256;
         const unsigned grid = (unsigned)std::min<long long>(need, 152 * 16);
         rc = brs_cuda_status(launch_pdl(scale_rows_kernel, dim3(grid), dim3(256), 0, s, bp, S->bs,
