@@ -27,6 +27,7 @@
 #include <utility>
 #include <vector>
 
+#include "dst_slices.cuh"
 #include "line_impl.cuh"
 #include "plane.cuh"
 #include "plane_tc.cuh"
@@ -105,6 +106,7 @@ struct PlaneState {
     void* tSeT = nullptr;    // transposes
     void* tSoT = nullptr;
     int fold = 1;            // BRSMOOTH_MODE_FOLD=0: the plain products
+    DstSlices* slices = nullptr;  // the same products on the tensor cores (dst_slices.cu)
 };
 
 // Map of a grid for the gather form, encoded on first use of its address.
@@ -714,6 +716,21 @@ int plane_pass(brs_ctx* c, const T* uin, T* uout, const T* b, int k0, int kstep,
     T* T2 = static_cast<T*>(P->t2);
     const T* Sx = static_cast<const T*>(P->sx);
     const T* Sy = static_cast<const T*>(P->sy);
+    if constexpr (sizeof(T) == 8) {
+        if (P->slices && P->form == 1) {
+            // R^ .* omega pv, the mode lines' solve, and the transform back with the update, both
+            // transforms on the tensor cores (256^3: 1.09 ms against 14.2 on the FP64 pipe)
+            int rc = dst_slices_rhs(P->slices, uin, b, c->p.az, T1,
+                                    static_cast<const double*>(P->tscale), ny, nz, k0, kstep,
+                                    nbatch, s);
+            if (rc == BRS_OK)
+                rc = mode_solve_launch(T1, T2, static_cast<const double*>(P->tfm),
+                                       static_cast<const double*>(P->tgm), nx, ny, nbatch, s);
+            return rc != BRS_OK ? rc
+                                : dst_slices_update(P->slices, T2, uin, 1.0 - c->omega, uout, ny,
+                                                    k0, kstep, nbatch, s);
+        }
+    }
     {
         const long long total = plane * nbatch;
         int blocks = (int)((total + 255) / 256);
@@ -1164,6 +1181,32 @@ int fused_setup(brs_ctx* c)
     return BRS_OK;
 }
 
+// S's even and odd rows on the first ceil(nx/2) / floor(nx/2) columns, and their transposes
+// (dst_fold_forward / _inverse).
+int fold_tables(PlaneState* P, int nx)
+{
+    const int Kd = nx / 2, Ks = nx - Kd;
+    const std::vector<double> S = dst1(nx);
+    std::vector<double> se((size_t)Ks * Ks), so((size_t)(Kd > 0 ? Kd : 1) * (Kd > 0 ? Kd : 1), 0.0);
+    std::vector<double> set(se.size()), sot(so.size(), 0.0);
+    for (int q = 0; q < Ks; ++q)
+        for (int x = 0; x < Ks; ++x) {
+            se[(size_t)q * Ks + x] = S[(size_t)(2 * q) * nx + x];
+            set[(size_t)x * Ks + q] = S[(size_t)(2 * q) * nx + x];
+        }
+    for (int q = 0; q < Kd; ++q)
+        for (int x = 0; x < Kd; ++x) {
+            so[(size_t)q * Kd + x] = S[(size_t)(2 * q + 1) * nx + x];
+            sot[(size_t)x * Kd + q] = S[(size_t)(2 * q + 1) * nx + x];
+        }
+    int rc = upload<double>(&P->tSe, se);
+    if (rc == BRS_OK)
+        rc = upload<double>(&P->tSo, so);
+    if (rc == BRS_OK)
+        rc = upload<double>(&P->tSeT, set);
+    return rc == BRS_OK ? upload<double>(&P->tSoT, sot) : rc;
+}
+
 // FP64 x-sine form with the twisted elimination: per-mode pivots of tridiag(-ay, d_p, -ay),
 // d_p = ax s_p + 2 ay + 2 az (twist_pivots, FP64), as the tables the kernel reads per step,
 // and the mode arrays; any ny.
@@ -1194,34 +1237,20 @@ int twist_setup(brs_ctx* c)
             e = cudaMemcpy(*dst, v.data(), v.size() * sizeof(double), cudaMemcpyHostToDevice);
         return brs_cuda_status(e);
     };
-    // S's even and odd rows on the first ceil(nx/2) / floor(nx/2) columns, and transposes
-    const int Kd = nx / 2, Ks = nx - Kd;
-    const std::vector<double> S = dst1(nx);
-    std::vector<double> se((size_t)Ks * Ks), so((size_t)(Kd > 0 ? Kd : 1) * (Kd > 0 ? Kd : 1), 0.0);
-    std::vector<double> set(se.size()), sot(so.size(), 0.0);
-    for (int q = 0; q < Ks; ++q)
-        for (int x = 0; x < Ks; ++x) {
-            se[(size_t)q * Ks + x] = S[(size_t)(2 * q) * nx + x];
-            set[(size_t)x * Ks + q] = S[(size_t)(2 * q) * nx + x];
-        }
-    for (int q = 0; q < Kd; ++q)
-        for (int x = 0; x < Kd; ++x) {
-            so[(size_t)q * Kd + x] = S[(size_t)(2 * q + 1) * nx + x];
-            sot[(size_t)x * Kd + q] = S[(size_t)(2 * q + 1) * nx + x];
-        }
     const char* fenv = std::getenv("BRSMOOTH_MODE_FOLD");
     P->fold = !(fenv && *fenv && std::atoi(fenv) == 0);
-    int rc = up(&P->tfm, fm);
+    int rc = BRS_OK;
+    // BRSMOOTH_MODE_SLICES=0 (or a choice among the FP64-pipe products, BRSMOOTH_MODE_FOLD)
+    // keeps the transforms off the tensor cores
+    const char* senv = std::getenv("BRSMOOTH_MODE_SLICES");
+    if (!fenv && !(senv && *senv && std::atoi(senv) == 0))
+        rc = dst_slices_create(nx, (long long)ny * p.nz, c->device, c->dev_status, &P->slices);
+    if (rc == BRS_OK)
+        rc = up(&P->tfm, fm);
     if (rc == BRS_OK)
         rc = up(&P->tfb, fb);
-    if (rc == BRS_OK)
-        rc = up(&P->tSe, se);
-    if (rc == BRS_OK)
-        rc = up(&P->tSo, so);
-    if (rc == BRS_OK)
-        rc = up(&P->tSeT, set);
-    if (rc == BRS_OK)
-        rc = up(&P->tSoT, sot);
+    if (rc == BRS_OK && !P->slices)
+        rc = fold_tables(P, nx);
     if (rc == BRS_OK)
         rc = up(&P->tgm, gm);
     if (rc == BRS_OK)
@@ -1260,7 +1289,15 @@ int twist_sweep(brs_ctx* c, void* u, const void* b, int nsweeps, cudaStream_t s,
     const double* Se = static_cast<const double*>(P->tSe);
     const double* So = static_cast<const double*>(P->tSo);
     int rc;
-    if (P->fold) {
+    const long long rows = (long long)ny * nz;
+    if (P->slices) {
+        rc = dst_slices_run(P->slices, static_cast<const double*>(b), mb,
+                            static_cast<const double*>(P->tscale), ny, rows, s);
+        if (rc == BRS_OK)
+            rc = u_zero ? brs_cuda_status(cudaMemsetAsync(mu, 0, (size_t)c->cells * sizeof(double), s))
+                        : dst_slices_run(P->slices, static_cast<const double*>(u), mu, nullptr, 1,
+                                         rows, s);
+    } else if (P->fold) {
         rc = dst_fold_forward(static_cast<const double*>(b), mb,
                               static_cast<const double*>(P->tscale), w1, Se, So, nx, ny, nz, s);
         if (rc == BRS_OK)
@@ -1295,6 +1332,8 @@ int twist_sweep(brs_ctx* c, void* u, const void* b, int nsweeps, cudaStream_t s,
             std::swap(cur, nxt);
         }
     }
+    if (rc == BRS_OK && P->slices)
+        return dst_slices_run(P->slices, cur, static_cast<double*>(u), nullptr, 1, rows, s);
     if (rc == BRS_OK)
         rc = P->fold ? dst_fold_inverse(cur, static_cast<double*>(u), w1, w2,
                                         static_cast<const double*>(P->tSeT),
@@ -1457,6 +1496,7 @@ void plane_teardown(brs_ctx* c)
                     P->tgb, P->tscale, P->mz, P->tSe, P->tSo, P->tSeT, P->tSoT})
         if (q)
             cudaFree(q);
+    dst_slices_destroy(P->slices);
     delete P;
     c->plane = nullptr;
 }

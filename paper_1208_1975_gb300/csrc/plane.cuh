@@ -19,6 +19,10 @@ int mode_twist_launch(const double* uin, double* out, double* zs, const double* 
                       const double* fm, const double* fb, const double* gm, const double* gb,
                       int nx, int ny, int nz, double omega, int colour, cudaStream_t s);
 
+// The block solve alone, out = M_p^{-1} r with r scaled by pv ([plane][y][p], out != r).
+int mode_solve_launch(const double* r, double* out, const double* fm, const double* gm, int nx,
+                      int ny, int planes, cudaStream_t s);
+
 // FP64 x-DST along the rows of [nz][ny][nx] arrays by the sine basis's even/odd symmetry
 // (plane_modes_f64.cu): out[k][y][p] = sum_x S[p][x] u[k][y][x] (times scale[y][p] if set),
 // and the inverse out[k][y][x] = sum_p S[x][p] uh[k][y][p].  Se / So: S's even / odd rows on

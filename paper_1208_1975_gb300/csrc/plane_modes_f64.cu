@@ -33,16 +33,16 @@ struct TwistModeArgs {
     double om1;          // 1 - omega
 };
 
-template <bool OMEGA1, int DF, int DB>
-__global__ void __launch_bounds__(256, 4) mode_twist_kernel(
+// ZC = false: no z coupling and no own value, out = M_p^{-1} b' (the block solve alone).
+template <bool OMEGA1, int DF, int DB, bool ZC>
+__global__ void __launch_bounds__(1024, 1) mode_twist_kernel(
     const double* uin, double* out, double* zs, const double* __restrict__ bs,
     const double* __restrict__ fm, const double* __restrict__ fb,
     const double* __restrict__ gm, const double* __restrict__ gb, const TwistModeArgs a)
 {
     pdl_wait_trigger();
-    const long long task = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    if (task >= a.ntasks)
-        return;  // warp-uniform
+    for (long long task = blockIdx.x + (long long)gridDim.x * (threadIdx.x >> 5); task < a.ntasks;
+         task += (long long)gridDim.x * (blockDim.x >> 5)) {
     const int lane = threadIdx.x & 31;
     const bool right = lane >= 16;
     const int n = a.ny, m = a.m, nx = a.nx;
@@ -65,10 +65,12 @@ __global__ void __launch_bounds__(256, 4) mode_twist_kernel(
         const long long o = base + (long long)y * nx;
         const bool q = on && ok;
         v.b = q ? __ldg(bs + o) : 0.0;
-        v.zn = (on && fzn) ? __ldg(uin + o - plane) : 0.0;
-        v.zp = (on && fzp) ? __ldg(uin + o + plane) : 0.0;
         v.f = q ? __ldg(fm + (long long)ss * nx + p) : 0.0;
-        v.g = q ? __ldg(fb + (long long)ss * nx + p) : 0.0;
+        if (ZC) {
+            v.zn = (on && fzn) ? __ldg(uin + o - plane) : 0.0;
+            v.zp = (on && fzp) ? __ldg(uin + o + plane) : 0.0;
+            v.g = q ? __ldg(fb + (long long)ss * nx + p) : 0.0;
+        }
     };
     // elimination towards the twist cell, DF cells of loads in flight
     double z = 0.0;
@@ -82,7 +84,7 @@ __global__ void __launch_bounds__(256, 4) mode_twist_kernel(
         for (int h = 0; h < DF; ++h) {
             const int ss = s + h;
             if (ss < cnt) {
-                const double r = fma(st[h].g, st[h].zn + st[h].zp, st[h].b);
+                const double r = ZC ? fma(st[h].g, st[h].zn + st[h].zp, st[h].b) : st[h].b;
                 z = fma(st[h].f, z, r);
                 if (ok)
                     zs[base + (long long)(right ? n - 1 - ss : ss) * nx] = z;
@@ -96,10 +98,14 @@ __global__ void __launch_bounds__(256, 4) mode_twist_kernel(
     if (!right) {
         const long long o = base + (long long)m * nx;
         const double bm = ok ? __ldg(bs + o) : 0.0;
-        const double zn = fzn ? __ldg(uin + o - plane) : 0.0;
-        const double zp = fzp ? __ldg(uin + o + plane) : 0.0;
-        const double gmv = ok ? __ldg(gm + p) : 0.0, gbv = ok ? __ldg(gb + p) : 0.0;
-        y = fma(gmv, z + zr, fma(gbv, zn + zp, bm));
+        const double gmv = ok ? __ldg(gm + p) : 0.0;
+        double r = bm;
+        if (ZC) {
+            const double zn = fzn ? __ldg(uin + o - plane) : 0.0;
+            const double zp = fzp ? __ldg(uin + o + plane) : 0.0;
+            r = fma(ok ? __ldg(gb + p) : 0.0, zn + zp, bm);
+        }
+        y = fma(gmv, z + zr, r);
         if (ok)
             out[o] = OMEGA1 ? y : fma(a.om1, uin[o], y);
     }
@@ -135,6 +141,7 @@ __global__ void __launch_bounds__(256, 4) mode_twist_kernel(
             loadb(h, ss + DB, ss + DB < cnt);
         }
     }
+    }  // task
 }
 
 // ---------------------------------------------------------------------------------------
@@ -285,6 +292,33 @@ cudaError_t launch_strided(const double* A, const double* B, double* C, const St
     return launch_pdl(gemm_strided_kernel, grid, dim3(256), 0, s, A, B, C, g);
 }
 
+using TwistModeKernel = void (*)(const double*, double*, double*, const double*, const double*,
+                                 const double*, const double*, const double*, const TwistModeArgs);
+
+// Grids of at least 20 warp tasks per SM: one CTA per SM with an equal share of them, in rounds
+// of at most 32 warps (256^3 has 27 tasks per SM, which 8-warp CTAs, four to an SM, spread as 24
+// or 32: 184 -> 158 us per Jacobi sweep).  Smaller ones keep 8-warp CTAs, which leave SMs free for
+// the next launch's prologue (128^3 calls of 50: 1.84 ms against 2.00 with one CTA per SM).
+int launch_twist(const TwistModeArgs& a, TwistModeKernel k, const double* uin, double* out,
+                 double* zs, const double* bs, const double* fm, const double* fb, const double* gm,
+                 const double* gb, cudaStream_t s)
+{
+    if (a.ntasks == 0)
+        return BRS_OK;
+    int dev = 0, sms = 1;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess)
+        e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess)
+        return brs_cuda_status(e);
+    const long long per_sm = (a.ntasks + sms - 1) / sms, rounds = (per_sm + 31) / 32;
+    const bool share = per_sm >= 20;
+    const int warps = share ? (int)((per_sm + rounds - 1) / rounds) : 8;
+    const unsigned grid = (unsigned)(share ? sms : (a.ntasks + 7) / 8);
+    e = launch_pdl(k, dim3(grid), dim3(32 * warps), 0, s, uin, out, zs, bs, fm, fb, gm, gb, a);
+    return brs_cuda_status(e);
+}
+
 unsigned row_grid(long long work)
 {
     long long b = (work + 255) / 256;
@@ -350,14 +384,22 @@ int mode_twist_launch(const double* uin, double* out, double* zs, const double* 
     const long long planes = colour < 0 ? nz : (nz - colour + 1) / 2;
     a.ntasks = planes * a.npb;
     a.om1 = 1.0 - omega;
-    if (a.ntasks == 0)
-        return BRS_OK;
-    const unsigned grid = (unsigned)((a.ntasks + 7) / 8);
-    cudaError_t e =
-        a.om1 == 0.0
-            ? launch_pdl(mode_twist_kernel<true, 2, 4>, dim3(grid), dim3(256), 0, s, uin, out, zs,
-                         bs, fm, fb, gm, gb, a)
-            : launch_pdl(mode_twist_kernel<false, 2, 4>, dim3(grid), dim3(256), 0, s, uin, out,
-                         zs, bs, fm, fb, gm, gb, a);
-    return brs_cuda_status(e);
+    return launch_twist(a, a.om1 == 0.0 ? mode_twist_kernel<true, 2, 4, true>
+                                        : mode_twist_kernel<false, 2, 4, true>,
+                        uin, out, zs, bs, fm, fb, gm, gb, s);
+}
+
+int mode_solve_launch(const double* r, double* out, const double* fm, const double* gm, int nx,
+                      int ny, int planes, cudaStream_t s)
+{
+    TwistModeArgs a{};
+    a.nx = nx;
+    a.ny = ny;
+    a.nz = planes;
+    a.m = (ny - 1) / 2;
+    a.npb = (nx + 15) / 16;
+    a.colour = -1;
+    a.ntasks = (long long)planes * a.npb;
+    return launch_twist(a, mode_twist_kernel<true, 2, 4, false>, nullptr, out, out, r, fm, nullptr,
+                        gm, nullptr, s);
 }
