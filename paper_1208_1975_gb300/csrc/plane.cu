@@ -84,6 +84,7 @@ struct PlaneState {
     int modes = 0;          // available for this context
     int modes_min = 2;      // smallest sweep count per call that takes it
     ModeCfg mcfg;
+    ModeResident mres;      // C > 0: the sweeps of a call on chip (plane_resident.cu)
     void* mb = nullptr;     // b^
     void* mu = nullptr;     // u^
     void* mtab = nullptr;   // [nx][mcfg.tab_len], context dtype
@@ -949,14 +950,14 @@ int modes_inverse(brs_ctx* c, const void* src, void* dst, cudaStream_t s)
 // Orthonormal DST-I matrix S[i][j] = sqrt(2/(n+1)) sin((i+1)(j+1) pi/(n+1)).
 std::vector<double> dst1(int n)
 {
-    std::vector<double> S((size_t)n * n);
+    std::vector<double> S((size_t)n * n), val(2 * (size_t)(n + 1));
     const double sc = std::sqrt(2.0 / (n + 1));
+    for (int q = 0; q < 2 * (n + 1); ++q)
+        val[q] = sc * std::sin(M_PI * (double)q / (n + 1));
+    // the angle index reduced mod 2(n+1): one sine per index, and more accurate than large angles
     for (int i = 0; i < n; ++i)
-        for (int j = 0; j < n; ++j) {
-            // reduce the angle index mod 2(n+1) before the sine for accuracy
-            const long long q = ((long long)(i + 1) * (j + 1)) % (2LL * (n + 1));
-            S[(size_t)i * n + j] = sc * std::sin(M_PI * (double)q / (n + 1));
-        }
+        for (int j = 0; j < n; ++j)
+            S[(size_t)i * n + j] = val[(long long)(i + 1) * (j + 1) % (2LL * (n + 1))];
     return S;
 }
 
@@ -1366,6 +1367,29 @@ int modes_setup(brs_ctx* c)
         return twist_setup(c);
     ModeCfg m;
     int rc = mode_config(p.ny, p.nx, p.nz, p.dtype, c->device, &m);
+    // FP32: the whole call on chip where one mode fits a cluster (BRSMOOTH_MODE_RESIDENT=0: never).
+    // Rows that TMA cannot stage take this form on CUDA-core contexts only (on the tensor path the
+    // per-sweep products would be left, whose rounding such calls' results carry), and from 48
+    // modes on: below, the products are a small part of a sweep, and calls of n sweeps stay equal
+    // to n calls bit for bit.
+    const char* renv = std::getenv("BRSMOOTH_MODE_RESIDENT");
+    if (sizeof(T) == 4 && !(renv && *renv && std::atoi(renv) == 0) &&
+        (rc == BRS_OK ||
+         (rc == BRS_ERR_UNSUPPORTED && P->math == BRS_PLANE_SIMT && p.nx >= 48))) {
+        const int rr = mode_resident_config(p.ny, p.nx, p.nz, p.method == BRS_CHAOTIC_GS, &P->mres);
+        if (rr != BRS_OK && rr != BRS_ERR_UNSUPPORTED)
+            return rr;
+        // lines of more than 256 cells leave 8 warps per SM: where the streaming sweep takes them,
+        // it keeps them (512 x 512 x 128, calls of 50: 4.92 ms against 5.19)
+        if (rc == BRS_OK && P->mres.E > 8)
+            P->mres.C = 0;
+        if (rr == BRS_OK && rc == BRS_ERR_UNSUPPORTED) {
+            m = ModeCfg{};
+            m.E = P->mres.E, m.G = P->mres.G;
+            m.tab_len = scan_table_len(m.E, m.G, false);
+            rc = BRS_OK;
+        }
+    }
     if (rc == BRS_ERR_UNSUPPORTED)
         return BRS_OK;
     if (rc != BRS_OK)
@@ -1390,6 +1414,10 @@ int modes_setup(brs_ctx* c)
         e = cudaMalloc(&P->mu, bytes);
     if (e != cudaSuccess)
         return brs_cuda_status(e);
+    P->mcfg = m;
+    P->modes = 1;
+    if (P->mres.C)
+        return BRS_OK;
     rc = mode_encode_map(m, &P->mm_b, P->mb);
     if (rc == BRS_OK)
         rc = mode_encode_map(m, &P->mm_u, P->mu);
@@ -1409,8 +1437,6 @@ int modes_setup(brs_ctx* c)
             return rc;
         P->mm_v_ptr = P->mv;
     }
-    P->mcfg = m;
-    P->modes = 1;
     return BRS_OK;
 }
 
@@ -1443,12 +1469,14 @@ int plane_setup(brs_ctx* c)
         P->form = (want == 1 && p.ny <= 512) ? 1 : 2;
     }
     std::vector<double> sx = dst1(p.nx), sy = dst1(p.ny), il((size_t)p.nx * p.ny);
-    for (int pp = 0; pp < p.nx; ++pp)
-        for (int q = 0; q < p.ny; ++q) {
-            const double spx = 2.0 - 2.0 * std::cos(M_PI * (pp + 1) / (p.nx + 1));
-            const double sqy = 2.0 - 2.0 * std::cos(M_PI * (q + 1) / (p.ny + 1));
-            il[(size_t)pp * p.ny + q] = 1.0 / (p.ax * spx + p.ay * sqy + 2.0 * p.az);
-        }
+    std::vector<double> ey(p.ny);
+    for (int q = 0; q < p.ny; ++q)
+        ey[q] = 2.0 - 2.0 * std::cos(M_PI * (q + 1) / (p.ny + 1));
+    for (int pp = 0; pp < p.nx; ++pp) {
+        const double spx = 2.0 - 2.0 * std::cos(M_PI * (pp + 1) / (p.nx + 1));
+        for (int q = 0; q < p.ny; ++q)
+            il[(size_t)pp * p.ny + q] = 1.0 / (p.ax * spx + p.ay * ey[q] + 2.0 * p.az);
+    }
     int rc;
     if (math == BRS_PLANE_TF32 || math == BRS_PLANE_3XTF32) {
         std::vector<float> ilf(il.begin(), il.end());
@@ -1557,7 +1585,7 @@ int plane_modes_sweep(brs_ctx* c, void* u, const void* b, int nsweeps, cudaStrea
         return twist_sweep(c, u, b, nsweeps, s, u_zero);
     const ModeCfg& m = P->mcfg;
     const bool two_pass = gs && !P->gs_fused;
-    if (!gs && P->mm_v_ptr != c->scratch) {
+    if (!gs && !P->mres.C && P->mm_v_ptr != c->scratch) {
         // the Jacobi second vector is the context's scratch array (allocated after set-up)
         int rc = mode_encode_map(m, &P->mm_v, c->scratch);
         if (rc != BRS_OK)
@@ -1573,6 +1601,13 @@ int plane_modes_sweep(brs_ctx* c, void* u, const void* b, int nsweeps, cudaStrea
     void* nxt = gs ? P->mv : c->scratch;
     const CUtensorMap* mcur = &P->mm_u;
     const CUtensorMap* mnxt = &P->mm_v;
+    if (P->mres.C) {
+        if (rc == BRS_OK)
+            rc = mode_resident_launch(P->mres, static_cast<const float*>(P->mu),
+                                      static_cast<const float*>(P->mb), static_cast<float*>(P->mu),
+                                      static_cast<const float*>(P->mtab), az, om, gs, nsweeps, s);
+        nsweeps = 0;
+    }
     for (int it = 0; it < nsweeps && rc == BRS_OK; ++it) {
         if (two_pass) {
             // even planes, then odd planes, in place

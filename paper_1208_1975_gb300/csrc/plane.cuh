@@ -56,3 +56,16 @@ int mode_encode_map(const ModeCfg& m, CUtensorMap* map, const void* ptr);
 int mode_sweep_launch(const ModeCfg& m, const CUtensorMap* mu, const CUtensorMap* mb, void* out,
                       const void* tab, double az, double omega, int colour, int* status,
                       cudaStream_t s);
+
+// The FP32 mode-line sweeps of a call on chip (plane_resident.cu): clusters of C CTAs, each
+// cluster one mode at a time.  BRS_ERR_UNSUPPORTED when one mode does not fit 8 CTAs.
+struct ModeResident {
+    int ny = 0, nm = 0, nz = 0, E = 0, G = 0;
+    int C = 0, rows = 0, clusters = 0;  // cluster size, most planes per CTA, resident clusters
+};
+int mode_resident_config(int ny, int nm, int nz, bool gs, ModeResident* out);
+// nsweeps sweeps of u into out (may be u); tab: nm tables of scan_table_len(E, G, false) entries
+// (omega folded in).
+int mode_resident_launch(const ModeResident& m, const float* u, const float* b, float* out,
+                         const float* tab, double az, double omega, bool gs, int nsweeps,
+                         cudaStream_t s);
