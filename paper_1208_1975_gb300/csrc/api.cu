@@ -208,16 +208,16 @@ PFN_encode_tiled brs_encoder()
     return reinterpret_cast<PFN_encode_tiled>(encoder());
 }
 
-const CUtensorMap* brs_tmap(brs_ctx* c, const void* ptr, int rows, int* rc)
+int brs_tmap(brs_ctx* c, const void* ptr, int rows, CUtensorMap* map)
 {
     for (auto& t : c->tmaps)
-        if (t.ptr == ptr && t.rows == rows)
-            return &t.map;
+        if (t.ptr == ptr && t.rows == rows) {
+            *map = t.map;
+            return BRS_OK;
+        }
     auto enc = encoder();
-    if (!enc) {
-        *rc = BRS_ERR_CUDA;
-        return nullptr;
-    }
+    if (!enc)
+        return BRS_ERR_CUDA;
     const brs_params& p = c->p;
     TmapEntry ent{};
     ent.ptr = ptr;
@@ -232,14 +232,13 @@ const CUtensorMap* brs_tmap(brs_ctx* c, const void* ptr, int rows, int* rc)
                      3, const_cast<void*>(ptr), gdim, gstride, box, estr,
                      CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
                      CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    if (r != CUDA_SUCCESS) {
-        *rc = BRS_ERR_CUDA;
-        return nullptr;
-    }
+    if (r != CUDA_SUCCESS)
+        return BRS_ERR_CUDA;
     if (c->tmaps.size() >= 16)
         c->tmaps.erase(c->tmaps.begin());
     c->tmaps.push_back(ent);
-    return &c->tmaps.back().map;
+    *map = ent.map;
+    return BRS_OK;
 }
 
 extern "C" {

@@ -139,8 +139,9 @@ typedef CUresult (*PFN_encode_tiled)(CUtensorMap*, CUtensorMapDataType, cuuint32
                                      CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 // cuTensorMapEncodeTiled from the driver (nullptr if unavailable).
 PFN_encode_tiled brs_encoder();
-// 3D tiled map over a grid array with box (bx, rows, 1); cached per (pointer, rows).
-const CUtensorMap* brs_tmap(brs_ctx* c, const void* ptr, int rows, int* rc);
+// 3D tiled map over a grid array with box (bx, rows, 1); cached per (pointer, rows), copied out
+// (the cache moves its entries when the next one comes in).
+int brs_tmap(brs_ctx* c, const void* ptr, int rows, CUtensorMap* map);
 
 // --------------------------------------------------------------------------------------
 // Device helpers: PTX wrappers for mbarrier + TMA, bounded waits.

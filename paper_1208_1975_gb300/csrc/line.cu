@@ -217,14 +217,12 @@ int line_sweep_launch(brs_ctx* c, const void* uin, void* uout, const void* b, cu
     a.status = c->dev_status;
     cudaError_t e;
     if (L.tma) {
-        int rc = BRS_OK;
-        const CUtensorMap* mu = brs_tmap(c, uin, L.JT + 2, &rc);
+        CUtensorMap tu, tbm;
+        int rc = brs_tmap(c, uin, L.JT + 2, &tu);
+        if (rc == BRS_OK)
+            rc = brs_tmap(c, b, L.JT, &tbm);
         if (rc != BRS_OK)
             return rc;
-        const CUtensorMap* mb = brs_tmap(c, b, L.JT, &rc);
-        if (rc != BRS_OK)
-            return rc;
-        CUtensorMap tu = *mu, tbm = *mb;
         void* out = uout;
         const void* tab = L.pair ? c->line_tab2 : c->line_tab;
         void* args[] = {&tu, &tbm, &out, (void*)&tab, &a};
