@@ -107,7 +107,10 @@ struct PlaneState {
     void* tSeT = nullptr;    // transposes
     void* tSoT = nullptr;
     int fold = 1;            // BRSMOOTH_MODE_FOLD=0: the plain products
-    DstSlices* slices = nullptr;  // the same products on the tensor cores (dst_slices.cu)
+    // the x-DST products by digits on the tensor cores (dst_slices.cu): the FP64 x-sine form, and
+    // FP32 contexts on CUDA cores
+    DstSlices<double>* slices = nullptr;
+    DstSlices<float>* slices32 = nullptr;
 };
 
 // Map of a grid for the gather form, encoded on first use of its address.
@@ -723,13 +726,28 @@ int plane_pass(brs_ctx* c, const T* uin, T* uout, const T* b, int k0, int kstep,
             // transforms on the tensor cores (256^3: 1.09 ms against 14.2 on the FP64 pipe)
             int rc = dst_slices_rhs(P->slices, uin, b, c->p.az, T1,
                                     static_cast<const double*>(P->tscale), ny, nz, k0, kstep,
-                                    nbatch, s);
+                                    nbatch, false, s);
             if (rc == BRS_OK)
                 rc = mode_solve_launch(T1, T2, static_cast<const double*>(P->tfm),
                                        static_cast<const double*>(P->tgm), nx, ny, nbatch, s);
             return rc != BRS_OK ? rc
-                                : dst_slices_update(P->slices, T2, uin, 1.0 - c->omega, uout, ny,
-                                                    k0, kstep, nbatch, s);
+                                : dst_slices_update(P->slices, T2, uin, 1.0 - c->omega, 1.0, uout,
+                                                    ny, k0, kstep, nbatch, s);
+        }
+    }
+    if constexpr (sizeof(T) == 4) {
+        if (P->slices32 && P->form == 1) {
+            // R^ [p][y], the y solve per x-mode, and the transform back with the update
+            int rc = dst_slices_rhs<float>(P->slices32, uin, b, c->p.az, T1, nullptr, ny, nz, k0,
+                                           kstep, nbatch, true, s);
+            if (rc != BRS_OK)
+                return rc;
+            const cudaError_t e = launch_ythomas<T, 0>(P, T1, nullptr, T2, nullptr, nx, ny, 0, 1,
+                                                       nbatch, s);
+            if (e != cudaSuccess)
+                return brs_cuda_status(e);
+            return dst_slices_update<float>(P->slices32, T2, uin, 1.0 - c->omega, c->omega, uout,
+                                            ny, k0, kstep, nbatch, s);
         }
     }
     {
@@ -865,6 +883,9 @@ int modes_forward(brs_ctx* c, const void* src, void* dst, cudaStream_t s)
     const int nx = c->p.nx, ny = c->p.ny, nz = c->p.nz;
     const long long plane = (long long)nx * ny;
     cudaError_t e;
+    if (P->slices32)
+        return dst_slices_to_modes(P->slices32, static_cast<const float*>(src),
+                                   static_cast<float*>(dst), ny, nz, s);
     if (modes_simt(c, P)) {
         GemmArgs g{};
         g.M = nx; g.N = ny; g.K = nx; g.strideA = 0; g.strideB = plane; g.strideC = plane;
@@ -905,6 +926,9 @@ int modes_inverse(brs_ctx* c, const void* src, void* dst, cudaStream_t s)
     const long long plane = (long long)nx * ny;
     const dim3 tgrid((unsigned)(((ny + 31) / 32) * ((nx + 31) / 32)), (unsigned)(nz < 65535 ? nz : 65535));
     cudaError_t e;
+    if (P->slices32)
+        return dst_slices_from_modes(P->slices32, static_cast<const float*>(src),
+                                     static_cast<float*>(dst), ny, nz, s);
     if (modes_simt(c, P)) {
         GemmArgs g{};
         g.M = ny; g.N = nx; g.K = nx; g.strideA = plane; g.strideB = 0; g.strideC = plane;
@@ -1296,7 +1320,7 @@ int twist_sweep(brs_ctx* c, void* u, const void* b, int nsweeps, cudaStream_t s,
                             static_cast<const double*>(P->tscale), ny, rows, s);
         if (rc == BRS_OK)
             rc = u_zero ? brs_cuda_status(cudaMemsetAsync(mu, 0, (size_t)c->cells * sizeof(double), s))
-                        : dst_slices_run(P->slices, static_cast<const double*>(u), mu, nullptr, 1,
+                        : dst_slices_run<double>(P->slices, static_cast<const double*>(u), mu, nullptr, 1,
                                          rows, s);
     } else if (P->fold) {
         rc = dst_fold_forward(static_cast<const double*>(b), mb,
@@ -1334,7 +1358,7 @@ int twist_sweep(brs_ctx* c, void* u, const void* b, int nsweeps, cudaStream_t s,
         }
     }
     if (rc == BRS_OK && P->slices)
-        return dst_slices_run(P->slices, cur, static_cast<double*>(u), nullptr, 1, rows, s);
+        return dst_slices_run<double>(P->slices, cur, static_cast<double*>(u), nullptr, 1, rows, s);
     if (rc == BRS_OK)
         rc = P->fold ? dst_fold_inverse(cur, static_cast<double*>(u), w1, w2,
                                         static_cast<const double*>(P->tSeT),
@@ -1348,6 +1372,8 @@ int twist_sweep(brs_ctx* c, void* u, const void* b, int nsweeps, cudaStream_t s,
 // with the context's omega folded in (factored once in FP64), the mode arrays and their
 // maps.  Leaves the form off (per-sweep form only) when BRSMOOTH_PLANE_MODES=0 or the y rows
 // cannot be staged by TMA.
+constexpr int kModesRaggedMin = 48;
+
 template <typename T>
 int modes_setup(brs_ctx* c)
 {
@@ -1375,7 +1401,8 @@ int modes_setup(brs_ctx* c)
     const char* renv = std::getenv("BRSMOOTH_MODE_RESIDENT");
     if (sizeof(T) == 4 && !(renv && *renv && std::atoi(renv) == 0) &&
         (rc == BRS_OK ||
-         (rc == BRS_ERR_UNSUPPORTED && P->math == BRS_PLANE_SIMT && p.nx >= 48))) {
+         (rc == BRS_ERR_UNSUPPORTED && P->math == BRS_PLANE_SIMT &&
+          p.nx >= kModesRaggedMin))) {
         const int rr = mode_resident_config(p.ny, p.nx, p.nz, p.method == BRS_CHAOTIC_GS, &P->mres);
         if (rr != BRS_OK && rr != BRS_ERR_UNSUPPORTED)
             return rr;
@@ -1408,10 +1435,16 @@ int modes_setup(brs_ctx* c)
     if (e == cudaSuccess)
         e = cudaMemcpy(P->mtab, all.data(), all.size() * sizeof(T), cudaMemcpyHostToDevice);
     const size_t bytes = (size_t)c->cells * sizeof(T);
-    if (e == cudaSuccess)
-        e = cudaMalloc(&P->mb, bytes);
-    if (e == cudaSuccess)
-        e = cudaMalloc(&P->mu, bytes);
+    if (P->slices32 && P->mres.C) {
+        // neither the digits' transforms nor the sweeps on chip use the per-sweep intermediates
+        P->mb = P->t1;
+        P->mu = P->t2;
+    } else {
+        if (e == cudaSuccess)
+            e = cudaMalloc(&P->mb, bytes);
+        if (e == cudaSuccess)
+            e = cudaMalloc(&P->mu, bytes);
+    }
     if (e != cudaSuccess)
         return brs_cuda_status(e);
     P->mcfg = m;
@@ -1468,17 +1501,21 @@ int plane_setup(brs_ctx* c)
         const int want = fenv ? std::atoi(fenv) : 1;
         P->form = (want == 1 && p.ny <= 512) ? 1 : 2;
     }
-    std::vector<double> sx = dst1(p.nx), sy = dst1(p.ny), il((size_t)p.nx * p.ny);
-    std::vector<double> ey(p.ny);
-    for (int q = 0; q < p.ny; ++q)
-        ey[q] = 2.0 - 2.0 * std::cos(M_PI * (q + 1) / (p.ny + 1));
-    for (int pp = 0; pp < p.nx; ++pp) {
-        const double spx = 2.0 - 2.0 * std::cos(M_PI * (pp + 1) / (p.nx + 1));
+    const std::vector<double> sx = dst1(p.nx), sy = dst1(p.ny);
+    auto inverse_eigenvalues = [&] {
+        std::vector<double> il((size_t)p.nx * p.ny), ey(p.ny);
         for (int q = 0; q < p.ny; ++q)
-            il[(size_t)pp * p.ny + q] = 1.0 / (p.ax * spx + p.ay * ey[q] + 2.0 * p.az);
-    }
+            ey[q] = 2.0 - 2.0 * std::cos(M_PI * (q + 1) / (p.ny + 1));
+        for (int pp = 0; pp < p.nx; ++pp) {
+            const double spx = 2.0 - 2.0 * std::cos(M_PI * (pp + 1) / (p.nx + 1));
+            for (int q = 0; q < p.ny; ++q)
+                il[(size_t)pp * p.ny + q] = 1.0 / (p.ax * spx + p.ay * ey[q] + 2.0 * p.az);
+        }
+        return il;
+    };
     int rc;
     if (math == BRS_PLANE_TF32 || math == BRS_PLANE_3XTF32) {
+        const std::vector<double> il = inverse_eigenvalues();
         std::vector<float> ilf(il.begin(), il.end());
         rc = brs_cuda_status(cudaMalloc(&P->ilam, ilf.size() * 4));
         if (rc == BRS_OK)
@@ -1494,14 +1531,22 @@ int plane_setup(brs_ctx* c)
             rc = modes_setup<float>(c);
         return rc;
     }
-    if (p.dtype == BRS_F64)
-        rc = upload<double>(&P->sx, sx);
-    else
-        rc = upload<float>(&P->sx, sx);
-    if (rc == BRS_OK)
-        rc = p.dtype == BRS_F64 ? upload<double>(&P->sy, sy) : upload<float>(&P->sy, sy);
-    if (rc == BRS_OK)
-        rc = p.dtype == BRS_F64 ? upload<double>(&P->ilam, il) : upload<float>(&P->ilam, il);
+    auto up = [&](void** dst, const std::vector<double>& v) {
+        return p.dtype == BRS_F64 ? upload<double>(dst, v) : upload<float>(dst, v);
+    };
+    rc = BRS_OK;
+    // FP32 on CUDA cores: the transforms by digits on the tensor cores, exact to FP32's rounding
+    // (BRSMOOTH_MODE_SLICES=0: products of FP32 multiply-adds)
+    const char* senv = std::getenv("BRSMOOTH_MODE_SLICES");
+    if (p.dtype == BRS_F32 && P->form == 1 && !(senv && *senv && std::atoi(senv) == 0))
+        rc = dst_slices_create(p.nx, (long long)p.ny * p.nz, c->device, c->dev_status, &P->slices32);
+    if (rc == BRS_OK && !P->slices32)
+        rc = up(&P->sx, sx);
+    if (rc == BRS_OK && P->form == 2) {
+        rc = up(&P->sy, sy);
+        if (rc == BRS_OK)
+            rc = up(&P->ilam, inverse_eigenvalues());
+    }
     const size_t bytes = (size_t)c->cells * c->esize;
     if (rc == BRS_OK)
         rc = brs_cuda_status(cudaMalloc(&P->t1, bytes));
@@ -1519,12 +1564,15 @@ void plane_teardown(brs_ctx* c)
     PlaneState* P = ps(c);
     if (!P)
         return;
+    if (P->mb == P->t1)
+        P->mb = P->mu = nullptr;  // the same arrays
     for (void* q : {P->sx, P->sy, P->ilam, P->t1, P->t2, P->sx_lo, P->sy_lo, P->t1_lo, P->t2_lo,
                     P->ytab, P->ym, P->mb, P->mu, P->mtab, P->mv, P->tfm, P->tfb, P->tgm,
                     P->tgb, P->tscale, P->mz, P->tSe, P->tSo, P->tSeT, P->tSoT})
         if (q)
             cudaFree(q);
     dst_slices_destroy(P->slices);
+    dst_slices_destroy(P->slices32);
     delete P;
     c->plane = nullptr;
 }

@@ -6,7 +6,7 @@ import numpy as np
 import pytest
 
 from brs_inputs import initial_guess, rhs
-from gpu_common import to_dev, to_np
+from gpu_common import TOL, rounded, to_dev, to_np
 from test_gpu_box import brs  # noqa: F401
 
 pytestmark = pytest.mark.gpu
@@ -38,6 +38,32 @@ def test_digits_equal_fp64_products(brs, shape, method, omega, nsweeps, monkeypa
     monkeypatch.setenv("BRSMOOTH_MODE_SLICES", "0")
     ref = sweep(brs, u, b, method, omega, nsweeps)
     assert np.max(np.abs(got - ref)) <= 1e-13 * np.max(np.abs(u))
+
+
+SHAPES32 = [(95, 7, 4), (96, 33, 5), (97, 5, 3), (128, 130, 3), (129, 4, 2), (200, 37, 9), (255, 3, 3),
+            (256, 6, 70), (300, 257, 2), (479, 5, 2), (100, 31, 200)]
+
+
+@pytest.mark.parametrize("nsweeps", [1, 3])
+@pytest.mark.parametrize("method,omega", [("jacobi", 0.8), ("gs", 1.0), ("gs", 1.3)])
+@pytest.mark.parametrize("shape", SHAPES32, ids=lambda s: "x".join(map(str, s)))
+def test_fp32_digits_equal_products(brs, shape, method, omega, nsweeps, monkeypatch):  # noqa: F811
+    """FP32 contexts on CUDA cores: each form is within the per-sweep tolerance of the exact sweep."""
+    nx, ny, nz = shape
+    u = rounded(initial_guess((nz, ny, nx)), "f32")
+    b = rounded(rhs((nz, ny, nx)), "f32")
+
+    def run():
+        with brs.Context(nx, ny, nz, (1.0, 0.5, 0.25), block="plane", method=method, dtype="f32",
+                         omega=omega, plane_math="simt") as ctx:
+            ut, bt = to_dev(u, "f32"), to_dev(b, "f32")
+            ctx.sweep(ut, bt, nsweeps)
+            assert ctx.last_error() == 0
+            return to_np(ut)
+
+    got = run()
+    monkeypatch.setenv("BRSMOOTH_MODE_SLICES", "0")
+    assert np.max(np.abs(got - run())) <= 2 * nsweeps * TOL["f32"] * np.max(np.abs(u))
 
 
 @pytest.mark.parametrize("scale", [1e-300, 1e-250, 1.0, 1e250, 1e300])
