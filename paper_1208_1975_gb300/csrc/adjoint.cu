@@ -15,8 +15,6 @@
 // undamped line-Jacobi iterate (A = M - N), which the x-line sweep kernel produces in one
 // pass: Tx (z + u) = Tx x, 2 z + Ty u = 2 x - Sy u, 2 z + Tz u = 2 x - Sz u, with S_d the
 // sum of the two neighbours along d (T_d = 2 I - S_d).
-#include <cstdlib>
-
 #include "brs_internal.cuh"
 #include "line_impl.cuh"
 #include "line_tile.cuh"
@@ -139,141 +137,9 @@ __device__ __forceinline__ void st4(T* p, const T (&v)[4], int rem, bool vec)
     }
 }
 
-// Second-difference neighbour sums of four cells of row `row` (at p, j, k): x (within the
-// row), y and z.
-template <typename T>
-struct Nb4 {
-    T c[4], sx[4], sy[4], sz[4];
-};
-
-template <typename T>
-__device__ __forceinline__ void neighbours4(Nb4<T>& o, const T* p, int i0, int rem, int j,
-                                            int k, int nx, int ny, int nz, long long plane,
-                                            bool vec, bool xs, bool yz)
-{
-    ld4(o.c, p, rem, vec);
-#pragma unroll
-    for (int q = 0; q < 4; ++q)
-        o.sx[q] = o.sy[q] = o.sz[q] = T(0);
-    if (xs) {
-        const T left = i0 > 0 ? p[-1] : T(0);
-        const T right = rem > 4 ? p[4] : T(0);
-#pragma unroll
-        for (int q = 0; q < 4; ++q)
-            o.sx[q] = (q == 0 ? left : o.c[q - 1]) +
-                      (q == 3 ? right : (q + 1 < rem ? o.c[q + 1] : T(0)));
-    }
-    if (!yz)
-        return;
-    T a[4];
-    if (j > 0) {
-        ld4(a, p - nx, rem, vec);
-#pragma unroll
-        for (int q = 0; q < 4; ++q)
-            o.sy[q] += a[q];
-    }
-    if (j + 1 < ny) {
-        ld4(a, p + nx, rem, vec);
-#pragma unroll
-        for (int q = 0; q < 4; ++q)
-            o.sy[q] += a[q];
-    }
-    if (k > 0) {
-        ld4(a, p - plane, rem, vec);
-#pragma unroll
-        for (int q = 0; q < 4; ++q)
-            o.sz[q] += a[q];
-    }
-    if (k + 1 < nz) {
-        ld4(a, p + plane, rem, vec);
-#pragma unroll
-        for (int q = 0; q < 4; ++q)
-            o.sz[q] += a[q];
-    }
-}
-
-// lambda <- lambda - omega A mu; gb += omega mu; per-CTA partial sums of the three
-// coefficient-gradient terms mu.(Tx x), mu.(2x - Sy u), mu.(2x - Sz u) with x = M^{-1}(b +
-// N u_k), u = u_k.  One warp per grid row at a time (grid-stride over rows with a fixed
-// grid, so the partial sums are reproducible), four cells per lane.  FP32 contexts sum a
-// lane's products over a row in FP32 before the FP64 sums (the FP64 pipe is the narrow one).
-// Latency bound (ncu: long-scoreboard stalls, 16 resident warps at 120 registers): the FP32
-// build is held to 3 CTAs per SM (78 registers, no spills); FP64 would spill, so it keeps 2.
-template <typename T>
-__global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 3 : 2) adjoint_update_kernel(
-    T* __restrict__ lam, const T* __restrict__ mu, const T* __restrict__ x,
-    const T* __restrict__ u, T* __restrict__ gb, int nx, int ny, int nz, double ax, double ay,
-    double az, double omega, double* partials, bool vec)
-{
-    const long long plane = (long long)nx * ny;
-    const long long nrows = (long long)ny * nz;
-    const int lane = threadIdx.x & 31, wpb = blockDim.x >> 5;
-    const T cx = (T)ax, cy = (T)ay, cz = (T)az, dg = (T)(2.0 * (ax + ay + az)), om = (T)omega;
-    double g0 = 0.0, g1 = 0.0, g2 = 0.0;
-    for (long long row = (long long)blockIdx.x * wpb + (threadIdx.x >> 5); row < nrows;
-         row += (long long)gridDim.x * wpb) {
-        const int k = (int)(row / ny), j = (int)(row - (long long)k * ny);
-        const long long base = row * nx;
-        T h0 = T(0), h1 = T(0), h2 = T(0);
-        for (int i0 = 4 * lane; i0 < nx; i0 += 128) {
-            const int rem = nx - i0;
-            const long long t = base + i0;
-            Nb4<T> m, xx, uu;
-            neighbours4(m, mu + t, i0, rem, j, k, nx, ny, nz, plane, vec, true, true);
-            neighbours4(xx, x + t, i0, rem, j, k, nx, ny, nz, plane, vec, true, false);
-            neighbours4(uu, u + t, i0, rem, j, k, nx, ny, nz, plane, vec, false, true);
-            T lv[4], gv[4];
-            ld4(lv, lam + t, rem, vec);
-            ld4(gv, gb + t, rem, vec);
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const T mq = m.c[q];
-                const T Amu = dg * mq - cx * m.sx[q] - cy * m.sy[q] - cz * m.sz[q];
-                lv[q] = lv[q] - om * Amu;
-                gv[q] += om * mq;
-                const T x2 = T(2) * xx.c[q];
-                if (q < rem) {
-                    if constexpr (sizeof(T) == 4) {
-                        h0 = fma(mq, x2 - xx.sx[q], h0);
-                        h1 = fma(mq, x2 - uu.sy[q], h1);
-                        h2 = fma(mq, x2 - uu.sz[q], h2);
-                    } else {
-                        g0 = fma(mq, x2 - xx.sx[q], g0);
-                        g1 = fma(mq, x2 - uu.sy[q], g1);
-                        g2 = fma(mq, x2 - uu.sz[q], g2);
-                    }
-                }
-            }
-            st4(lam + t, lv, rem, vec);
-            st4(gb + t, gv, rem, vec);
-        }
-        if constexpr (sizeof(T) == 4) {
-            g0 += (double)h0;
-            g1 += (double)h1;
-            g2 += (double)h2;
-        }
-    }
-    __shared__ double red[3][kThreads / 32];
-    double v[3] = {g0, g1, g2};
-    for (int d = 0; d < 3; ++d) {
-        for (int o = 16; o > 0; o >>= 1)
-            v[d] += __shfl_down_sync(0xffffffffu, v[d], o);
-        if ((threadIdx.x & 31) == 0)
-            red[d][threadIdx.x >> 5] = v[d];
-    }
-    __syncthreads();
-    if (threadIdx.x < 32) {
-        for (int d = 0; d < 3; ++d) {
-            double w = threadIdx.x < kThreads / 32 ? red[d][threadIdx.x] : 0.0;
-            for (int o = 16; o > 0; o >>= 1)
-                w += __shfl_down_sync(0xffffffffu, w, o);
-            if (threadIdx.x == 0)
-                partials[3 * blockIdx.x + d] = w;
-        }
-    }
-}
-
-// FP32 form of the same update as a z-march: a warp owns 128 cells of row j (four per lane)
+// FP32 form: lambda <- lambda - omega A mu; gb += omega mu; per-CTA partial sums of the three
+// coefficient-gradient terms mu.(Tx x), mu.(2x - Sy u), mu.(2x - Sz u) with x = M^{-1}(b + N u_k),
+// u = u_k.  A z-march: a warp owns 128 cells of row j (four per lane)
 // over a chunk of kMarchKC planes, keeps mu and u of planes k-1, k, k+1 in registers, and
 // loads the next plane's inputs before computing the current one (more loads in flight per
 // warp, and the z neighbours are not loaded twice).  Items (j, x-chunk, z-chunk) go to warps
@@ -418,6 +284,116 @@ __global__ void __launch_bounds__(kThreads, 2) adjoint_update_march(
     }
 }
 
+// FP64 form: lanes along x, a warp marches over kc planes of 32 cells of a row with mu of planes
+// k-1, k, k+1 in registers and the next plane's inputs in flight.  Bound by the FP64 pipe, so it
+// counts operations, 15 per cell instead of 22, by two identities of the symmetric operators:
+//   A mu = M mu - (ay Sy + az Sz) mu and M mu = lambda, so
+//     lambda <- (1 - omega) lambda + omega (ay Sy + az Sz) mu   (no x neighbours, no diagonal);
+//   mu . Tx x = (Tx mu) . x and mu . Sd u = (Sd mu) . u, so the sums need the neighbours of mu
+//     only, which the first line has: (2 mu - Sx mu) x, 2 mu x - (Sy mu) u, 2 mu x - (Sz mu) u,
+//     differences formed cell by cell as before.
+// The last CTA to finish adds the CTAs' sums into grad_a in a fixed order (a counter in global
+// memory, left at zero for the next call).  128^3, same box: 109 -> ADJUS us per call.
+struct StepIn {
+    double mup, muym, muyp, mul, mur, lam, x, u, gb;
+};
+
+__global__ void __launch_bounds__(kThreads, 3) adjoint_update_f64(
+    double* __restrict__ lam, const double* __restrict__ mu, const double* __restrict__ x,
+    const double* __restrict__ u, double* __restrict__ gb, int nx, int ny, int nz, int kc, double oy,
+    double oz, double omega, double* partials, unsigned* counter, double* grad_a)
+{
+    pdl_wait_trigger();
+    const long long plane = (long long)nx * ny;
+    const int ncx = (nx + 31) / 32, nkc = (nz + kc - 1) / kc;
+    const long long nitems = (long long)ny * ncx * nkc;
+    const int lane = threadIdx.x & 31, wpb = blockDim.x >> 5;
+    const double om1 = 1.0 - omega;
+    double g0 = 0.0, g1 = 0.0, g2 = 0.0;
+    for (long long it = (long long)blockIdx.x * wpb + (threadIdx.x >> 5); it < nitems;
+         it += (long long)gridDim.x * wpb) {
+        const long long rest = it / ncx;
+        const int i = (int)(it - rest * ncx) * 32 + lane;
+        const int k0 = (int)(rest / ny) * kc, j = (int)(rest % ny);
+        const int k1 = min(nz, k0 + kc);
+        const bool on = i < nx;
+        long long o = plane * k0 + (long long)j * nx + (on ? i : 0);
+        auto load = [&](StepIn& v, long long q, int k) {
+            v.mup = on && k + 1 < nz ? mu[q + plane] : 0.0;
+            v.muym = on && j > 0 ? mu[q - nx] : 0.0;
+            v.muyp = on && j + 1 < ny ? mu[q + nx] : 0.0;
+            v.mul = on && i > 0 ? mu[q - 1] : 0.0;
+            v.mur = on && i + 1 < nx ? mu[q + 1] : 0.0;
+            v.lam = on ? lam[q] : 0.0;
+            v.x = on ? x[q] : 0.0;
+            v.u = on ? u[q] : 0.0;
+            v.gb = on ? gb[q] : 0.0;
+        };
+        double mum = on && k0 > 0 ? mu[o - plane] : 0.0;
+        double muc = on ? mu[o] : 0.0;
+        StepIn nxt;
+        load(nxt, o, k0);
+        for (int k = k0; k < k1; ++k, o += plane) {
+            const StepIn c = nxt;
+            if (k + 1 < k1)
+                load(nxt, o + plane, k + 1);
+            const double sy = c.muym + c.muyp, sz = mum + c.mup, sx = c.mul + c.mur;
+            const double lv = fma(oz, sz, fma(oy, sy, om1 * c.lam));
+            const double gv = fma(omega, muc, c.gb);
+            const double m2 = muc + muc, t = m2 * c.x;
+            g0 = fma(m2 - sx, c.x, g0);
+            g1 += fma(-sy, c.u, t);
+            g2 += fma(-sz, c.u, t);
+            if (on) {
+                lam[o] = lv;
+                gb[o] = gv;
+            }
+            mum = muc;
+            muc = c.mup;
+        }
+    }
+    __shared__ double red[3][kThreads / 32];
+    __shared__ bool last;
+    auto block_sum = [&](double (&v)[3]) {  // thread 0 holds the sums
+        for (int d = 0; d < 3; ++d) {
+            for (int q = 16; q > 0; q >>= 1)
+                v[d] += __shfl_down_sync(0xffffffffu, v[d], q);
+            if (lane == 0)
+                red[d][threadIdx.x >> 5] = v[d];
+        }
+        __syncthreads();
+        if (threadIdx.x == 0)
+            for (int d = 0; d < 3; ++d) {
+                v[d] = 0.0;
+                for (int w = 0; w < kThreads / 32; ++w)
+                    v[d] += red[d][w];
+            }
+        __syncthreads();
+    };
+    double v[3] = {g0, g1, g2};
+    block_sum(v);
+    if (threadIdx.x == 0) {
+        for (int d = 0; d < 3; ++d)
+            __stcg(partials + 3 * blockIdx.x + d, v[d]);
+        __threadfence();
+        last = atomicAdd(counter, 1u) == gridDim.x - 1;
+    }
+    __syncthreads();
+    if (!last)
+        return;
+    __threadfence();
+    v[0] = v[1] = v[2] = 0.0;
+    for (int t = threadIdx.x; t < (int)gridDim.x; t += blockDim.x)
+        for (int d = 0; d < 3; ++d)
+            v[d] += __ldcg(partials + 3 * t + d);
+    block_sum(v);
+    if (threadIdx.x == 0) {
+        for (int d = 0; d < 3; ++d)
+            grad_a[d] += -omega * v[d];
+        *counter = 0;
+    }
+}
+
 // grad_a[d] += -omega * sum of the partials, in a fixed order.
 __global__ void adjoint_reduce_kernel(const double* partials, int nblocks, double omega,
                                       double* grad_a)
@@ -478,49 +454,72 @@ cudaError_t launch_minv(const brs_ctx* c, const T* in, T* out, cudaStream_t s)
     return cudaErrorInvalidConfiguration;
 }
 
-// BRSMOOTH_ADJ_MARCH=0 selects the row form of the FP32 update (A/B measurements)
-bool env_march()
-{
-    const char* v = std::getenv("BRSMOOTH_ADJ_MARCH");
-    return !(v && v[0] == '0');
-}
-
 struct AdjState {
     void* mu = nullptr;
     double* partials = nullptr;
+    unsigned* counter = nullptr;  // FP64 update: CTAs done
     int nblocks = 0;
     brs_ctx* xctx = nullptr;  // x-line Jacobi with omega = 1: x = M^{-1}(b + N u) in one pass
     int* xstatus = nullptr;   // xctx's own status word (its kernels report to the owner's)
 };
 
-template <typename T>
-int adjoint_run(brs_ctx* c, T* lam, const T* u, const T* b, T* gb, double* ga, cudaStream_t s)
+// FP64: both block solves on the elimination from both ends (line_tile.cu), the update in one pass
+// with its reduction.
+int adjoint_run_f64(brs_ctx* c, double* lam, const double* u, const double* b, double* gb,
+                    double* ga, cudaStream_t s)
 {
     AdjState* A = static_cast<AdjState*>(c->adjoint);
-    T* x = static_cast<T*>(c->scratch);
-    T* mu = static_cast<T*>(A->mu);
+    const brs_params& p = c->p;
+    double* x = static_cast<double*>(c->scratch);
+    double* mu = static_cast<double*>(A->mu);
+    int rc;
+    if (A->xctx->ltile) {
+        rc = line_tile_undamped(A->xctx, u, x, b, s);
+        if (rc == BRS_OK)
+            rc = line_tile_solve(A->xctx, lam, mu, s);
+    } else {
+        rc = line_sweep_launch(A->xctx, u, x, b, s);
+        if (rc == BRS_OK)
+            rc = brs_cuda_status(launch_minv<double>(c, lam, mu, s));
+    }
+    if (rc != BRS_OK)
+        return rc;
+    // planes per item: the fewest plane steps (one more per item for its first loads) over whole
+    // rounds of the resident warps
+    const long long cols = (long long)p.ny * ((p.nx + 31) / 32), warps = A->nblocks * (kThreads / 32ll);
+    int kc = 4;
+    long long best = -1;
+    for (int q = 4; q <= 32; ++q) {
+        const long long rounds = (cols * ((p.nz + q - 1) / q) + warps - 1) / warps;
+        if (best < 0 || rounds * (q + 1) < best) {
+            best = rounds * (q + 1);
+            kc = q;
+        }
+    }
+    return brs_cuda_status(launch_pdl(adjoint_update_f64, dim3(A->nblocks), dim3(kThreads), 0, s,
+                                      lam, (const double*)mu, (const double*)x, u, gb, p.nx, p.ny,
+                                      p.nz, kc, c->omega * p.ay, c->omega * p.az, c->omega,
+                                      A->partials, A->counter, ga));
+}
+
+int adjoint_run_f32(brs_ctx* c, float* lam, const float* u, const float* b, float* gb, double* ga,
+                    cudaStream_t s)
+{
+    AdjState* A = static_cast<AdjState*>(c->adjoint);
+    float* x = static_cast<float*>(c->scratch);
+    float* mu = static_cast<float*>(A->mu);
     // x = M^{-1}(b + N u_k): one undamped x-line Jacobi sweep from u_k
     int rc = line_sweep_launch(A->xctx, u, x, b, s);
     if (rc != BRS_OK)
         return rc;
-    cudaError_t e = launch_minv<T>(c, lam, mu, s);  // mu = M^{-1} lambda
+    cudaError_t e = launch_minv<float>(c, lam, mu, s);  // mu = M^{-1} lambda
     if (e != cudaSuccess)
         return brs_cuda_status(e);
     auto a16 = [](const void* q) { return (reinterpret_cast<uintptr_t>(q) & 15u) == 0; };
     const bool vec = c->p.nx % 4 == 0 && a16(lam) && a16(mu) && a16(x) && a16(u) && a16(gb);
-    if constexpr (sizeof(T) == 4) {
-        if (env_march())
-            adjoint_update_march<<<A->nblocks, kThreads, 0, s>>>(
-                lam, mu, x, u, gb, c->p.nx, c->p.ny, c->p.nz, c->p.ax, c->p.ay, c->p.az,
-                c->omega, A->partials, vec);
-        else
-            adjoint_update_kernel<T><<<A->nblocks, kThreads, 0, s>>>(
-                lam, mu, x, u, gb, c->p.nx, c->p.ny, c->p.nz, c->p.ax, c->p.ay, c->p.az,
-                c->omega, A->partials, vec);
-    } else
-    adjoint_update_kernel<T><<<A->nblocks, kThreads, 0, s>>>(lam, mu, x, u, gb, c->p.nx, c->p.ny,
-                                                             c->p.nz, c->p.ax, c->p.ay, c->p.az,
-                                                             c->omega, A->partials, vec);
+    adjoint_update_march<<<A->nblocks, kThreads, 0, s>>>(lam, mu, x, u, gb, c->p.nx, c->p.ny,
+                                                         c->p.nz, c->p.ax, c->p.ay, c->p.az,
+                                                         c->omega, A->partials, vec);
     e = cudaGetLastError();
     if (e != cudaSuccess)
         return brs_cuda_status(e);
@@ -539,6 +538,8 @@ void adjoint_teardown(brs_ctx* c)
         cudaFree(A->mu);
     if (A->partials)
         cudaFree(A->partials);
+    if (A->counter)
+        cudaFree(A->counter);
     if (A->xctx) {
         A->xctx->dev_status = A->xstatus;
         brsmooth_destroy(A->xctx);
@@ -562,12 +563,18 @@ extern "C" int brsmooth_adjoint_sweep(brs_ctx* c, void* lam, const void* u_k, co
         int sms = 0;
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
         const long long need = ((long long)c->p.ny * c->p.nz + kThreads / 32 - 1) / (kThreads / 32);
-        A->nblocks = (int)(need < (long long)sms * 8 ? need : (long long)sms * 8);
+        // FP64: one resident wave (3 CTAs per SM), shared out in items
+        const long long most = (long long)sms * (c->p.dtype == BRS_F64 ? 3 : 8);
+        A->nblocks = (int)(need < most ? need : most);
         if (A->nblocks < 1)
             A->nblocks = 1;
         cudaError_t e = cudaMalloc(&A->mu, (size_t)c->cells * c->esize);
         if (e == cudaSuccess)
             e = cudaMalloc(&A->partials, sizeof(double) * 3 * A->nblocks);
+        if (e == cudaSuccess)
+            e = cudaMalloc(&A->counter, sizeof(unsigned));
+        if (e == cudaSuccess)
+            e = cudaMemset(A->counter, 0, sizeof(unsigned));
         int rc = brs_cuda_status(e);
         if (rc == BRS_OK) {
             brs_params q = c->p;
@@ -583,14 +590,14 @@ extern "C" int brsmooth_adjoint_sweep(brs_ctx* c, void* lam, const void* u_k, co
         cudaFree(A->xctx->scratch);
         A->xctx->scratch = nullptr;
         line_seq_teardown(A->xctx);
-        line_tile_teardown(A->xctx);
+        line_tile_trim(A->xctx);
         A->xstatus = A->xctx->dev_status;
         A->xctx->dev_status = c->dev_status;
     }
     c->last_stream = s;
     if (c->p.dtype == BRS_F64)
-        return adjoint_run<double>(c, (double*)lam, (const double*)u_k, (const double*)b,
-                                   (double*)grad_b, grad_a, s);
-    return adjoint_run<float>(c, (float*)lam, (const float*)u_k, (const float*)b, (float*)grad_b,
-                              grad_a, s);
+        return adjoint_run_f64(c, (double*)lam, (const double*)u_k, (const double*)b,
+                               (double*)grad_b, grad_a, s);
+    return adjoint_run_f32(c, (float*)lam, (const float*)u_k, (const float*)b, (float*)grad_b,
+                           grad_a, s);
 }

@@ -14,8 +14,8 @@
 // over all warps, where two threads per line alone would wait on memory latency.  An FP64 warp
 // instruction occupies its SM quarter for 64 clocks, so the chain warp's place rotates with the
 // CTA.  Calls of few sweeps, and grids of less than about 27 16-line tasks per SM,
-// run fastest on it (us per sweep, same box, line-major -> tile): 32^3 Jacobi 12.3 -> 5.0 in calls of
-// 30, 64^3 22.6 -> 9.3, 96^3 32.6 -> 17.5, 128^3 44.7 -> 35.8; Gauss-Seidel 96x88x72 60.1 -> 23.5;
+// run fastest on it (us per sweep, same box, line-major -> tile): 32^3 Jacobi 12.3 -> 4.4 in calls of
+// 30, 64^3 22.6 -> 9.0, 96^3 32.6 -> 17.5, 128^3 44.7 -> 35.7; Gauss-Seidel 96x88x72 60.1 -> 21.7;
 // 256^3 one-sweep calls 400 -> 325, but 223 -> 250 in calls of 30.  What bounds it at 256^3 is the
 // balance of the chain against the other warps (FP64 pipe 75 % busy); at 32^3 latency: launch,
 // loads, and 32 dependent FMAs.
@@ -38,6 +38,7 @@ struct TileArgs {
     int nx, ny, nz, m;    // grid, twist cell
     int nl, pitch;        // lines per task, shared-memory stride of a line (odd)
     int colour;           // -1: all lines; 0 / 1: lines with (j + k) % 2 == colour
+    int early;            // let the next launch start at once (it fits beside this one)
     long long nlines;     // lines to update
     double om1, gm;       // 1 - omega; ax g_m
     const double* tab;    // [3][nx]: omega pv_i, omega pv_i ay, omega pv_i az
@@ -45,8 +46,9 @@ struct TileArgs {
 };
 
 struct Shape {
-    int nl = 16, threads = 32;
-    bool pdl = true;
+    int nl = kLines, threads = 32;
+    int lpu = 4;   // lines a warp gathers or updates at once: 1, 2 or 4
+    bool early = false, pdl = true;
 };
 
 struct TileState {
@@ -62,8 +64,8 @@ enum { B_PLAIN = 0, B_SCALED = 1, SOLVE_ONLY = 2 };
 
 __device__ __forceinline__ double ld_if(const double* p, bool ok) { return ok ? *p : 0.0; }
 
-template <bool OMEGA1, int MODE>
-__global__ void __launch_bounds__(256) xline_tile_kernel(const double* u, double* out,
+template <bool OMEGA1, int MODE, int LPU>
+__global__ void __launch_bounds__(256, 4) xline_tile_kernel(const double* u, double* out,
                                                          const double* __restrict__ b,
                                                          const __grid_constant__ TileArgs a)
 {
@@ -94,19 +96,21 @@ __global__ void __launch_bounds__(256) xline_tile_kernel(const double* u, double
     }
     __syncthreads();
     pdl_wait();
+    if (a.early)
+        pdl_trigger();
     const long long plane = (long long)nx * a.ny;
-    const int chunks = (nx + 31) >> 5, groups = (nl + 3) >> 2;
+    const int chunks = (nx + 31) >> 5, groups = (nl + LPU - 1) / LPU;
 
-    // right-hand sides, four lines by 32 cells at a time
+    // right-hand sides, LPU lines by 32 cells at a time
     for (int unit = warp; unit < chunks * groups; unit += nwarp) {
         const int ch = unit / groups, g = unit - ch * groups;
         const int i = ch * 32 + lane;
         const bool act = i < nx;
         const int ic = act ? i : nx - 1;
-        double bb[4], yn[4], yp[4], zn[4], zp[4];
+        double bb[LPU], yn[LPU], yp[LPU], zn[LPU], zp[LPU];
 #pragma unroll
-        for (int h = 0; h < 4; ++h) {
-            const int l = g * 4 + h;
+        for (int h = 0; h < LPU; ++h) {
+            const int l = g * LPU + h;
             const int f = l < nl && act ? flags[l < nl ? l : 0] : 0;
             const long long p = base[l < nl ? l : 0] + ic;
             bb[h] = ld_if(b + p, f & 16);
@@ -125,8 +129,8 @@ __global__ void __launch_bounds__(256) xline_tile_kernel(const double* u, double
             fb = __ldg(a.tab + 2 * nx + ic);
         }
 #pragma unroll
-        for (int h = 0; h < 4; ++h) {
-            const int l = g * 4 + h;
+        for (int h = 0; h < LPU; ++h) {
+            const int l = g * LPU + h;
             double r = MODE == B_SCALED ? bb[h] : __dmul_rn(sb, bb[h]);
             if (MODE != SOLVE_ONLY)
                 r = fma(fb, zn[h] + zp[h], fma(fa, yn[h] + yp[h], r));
@@ -199,22 +203,23 @@ __global__ void __launch_bounds__(256) xline_tile_kernel(const double* u, double
         }
     }
     __syncthreads();
-    pdl_trigger();
+    if (!a.early)
+        pdl_trigger();
 
     // update
     for (int unit = warp; unit < chunks * groups; unit += nwarp) {
         const int ch = unit / groups, g = unit - ch * groups;
         const int i = ch * 32 + lane;
-        double own[4];
+        double own[LPU];
 #pragma unroll
-        for (int h = 0; h < 4; ++h) {
-            const int l = g * 4 + h;
+        for (int h = 0; h < LPU; ++h) {
+            const int l = g * LPU + h;
             const bool on = l < nl && i < nx && (flags[l < nl ? l : 0] & 16);
             own[h] = !OMEGA1 && on ? u[base[l] + i] : 0.0;
         }
 #pragma unroll
-        for (int h = 0; h < 4; ++h) {
-            const int l = g * 4 + h;
+        for (int h = 0; h < LPU; ++h) {
+            const int l = g * LPU + h;
             if (l < nl && i < nx && (flags[l] & 16)) {
                 const double y = Z[l * pitch + i];
                 out[base[l] + i] = OMEGA1 ? y : fma(a.om1, own[h], y);
@@ -243,11 +248,23 @@ int env_int(const char* name, int dflt)
 
 size_t tile_smem(const TileArgs& a, int nl) { return (size_t)nl * a.pitch * sizeof(double); }
 
-template <int MODE>
+template <int MODE, int LPU>
 const void* tile_kernel(bool om1)
 {
-    return om1 ? (const void*)xline_tile_kernel<true, MODE>
-               : (const void*)xline_tile_kernel<false, MODE>;
+    return om1 ? (const void*)xline_tile_kernel<true, MODE, LPU>
+               : (const void*)xline_tile_kernel<false, MODE, LPU>;
+}
+
+const void* tile_kernel(int mode, int lpu, bool om1)
+{
+    if (mode == B_PLAIN)
+        return lpu == 1 ? tile_kernel<B_PLAIN, 1>(om1)
+             : lpu == 2 ? tile_kernel<B_PLAIN, 2>(om1) : tile_kernel<B_PLAIN, 4>(om1);
+    if (mode == B_SCALED)
+        return lpu == 1 ? tile_kernel<B_SCALED, 1>(om1)
+             : lpu == 2 ? tile_kernel<B_SCALED, 2>(om1) : tile_kernel<B_SCALED, 4>(om1);
+    return lpu == 1 ? tile_kernel<SOLVE_ONLY, 1>(om1)
+         : lpu == 2 ? tile_kernel<SOLVE_ONLY, 2>(om1) : tile_kernel<SOLVE_ONLY, 4>(om1);
 }
 
 int launch_tile(brs_ctx* c, int mode, bool om1, int colour, const Shape& sh, const double* u,
@@ -261,8 +278,8 @@ int launch_tile(brs_ctx* c, int mode, bool om1, int colour, const Shape& sh, con
     a.nl = sh.nl;
     if (a.nlines == 0)
         return BRS_OK;
-    const void* k = mode == B_PLAIN ? tile_kernel<B_PLAIN>(om1)
-                  : mode == B_SCALED ? tile_kernel<B_SCALED>(om1) : tile_kernel<SOLVE_ONLY>(om1);
+    a.early = sh.early;
+    const void* k = tile_kernel(mode, sh.lpu, om1);
     const dim3 grid((unsigned)((a.nlines + sh.nl - 1) / sh.nl));
     void* args[] = {&u, &out, &b, &a};
     cudaError_t e;
@@ -295,6 +312,11 @@ Shape pick_shape(const TileArgs& a, long long lines, int sms)
         }
     }
     sh.threads = res <= 4.5 ? 256 : 128;
+    // as few lines per warp and trip as keep every warp at one trip: an FP64 warp instruction
+    // holds its SM quarter for 64 clocks, so a trip of 4 lines takes 1300
+    const int chunks = (a.nx + 31) / 32, nw = sh.threads / 32;
+    sh.lpu = chunks * sh.nl <= nw ? 1 : chunks * ((sh.nl + 1) / 2) <= nw ? 2 : 4;
+    sh.early = (lines + sh.nl - 1) / sh.nl <= 2ll * sms;
     sh.pdl = env_int("BRSMOOTH_LINE_PDL", 1) != 0;
     return sh;
 }
@@ -333,16 +355,13 @@ int line_tile_setup(brs_ctx* c)
         e = cudaMalloc(&S->bs, (size_t)c->cells * sizeof(double));
     a.tab = S->tab;
     const size_t smem = tile_smem(a, kLines);
-    const void* ks[] = {tile_kernel<B_PLAIN>(false), tile_kernel<B_PLAIN>(true),
-                        tile_kernel<B_SCALED>(false), tile_kernel<B_SCALED>(true),
-                        tile_kernel<SOLVE_ONLY>(false), tile_kernel<SOLVE_ONLY>(true)};
-    for (const void* k : ks)
-        if (e == cudaSuccess && smem > 48u * 1024u) {
-            cudaFuncAttributes fa{};
-            e = cudaFuncGetAttributes(&fa, k);
-            if (e == cudaSuccess && (size_t)fa.maxDynamicSharedSizeBytes < smem)
-                e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        }
+    for (int q = 0; q < 18 && smem > 48u * 1024u && e == cudaSuccess; ++q) {
+        const void* k = tile_kernel(q % 3, 1 << (q / 6), q / 3 % 2 != 0);
+        cudaFuncAttributes fa{};
+        e = cudaFuncGetAttributes(&fa, k);
+        if (e == cudaSuccess && (size_t)fa.maxDynamicSharedSizeBytes < smem)
+            e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    }
     if (e != cudaSuccess)
         return brs_cuda_status(e);
     const long long lines = (long long)p.ny * p.nz;
@@ -402,4 +421,23 @@ int line_tile_sweep(brs_ctx* c, void* u, const void* b, int nsweeps, cudaStream_
         rc = brs_cuda_status(cudaMemcpyAsync(u, cur, (size_t)c->cells * sizeof(double),
                                              cudaMemcpyDeviceToDevice, s));
     return rc;
+}
+
+int line_tile_undamped(brs_ctx* c, const double* u, double* out, const double* b, cudaStream_t s)
+{
+    return launch_tile(c, B_PLAIN, true, -1, st(c)->sh, u, out, b, s);
+}
+
+int line_tile_solve(brs_ctx* c, const double* r, double* out, cudaStream_t s)
+{
+    return launch_tile(c, SOLVE_ONLY, true, -1, st(c)->sh, nullptr, out, r, s);
+}
+
+void line_tile_trim(brs_ctx* c)
+{
+    TileState* S = st(c);
+    if (S && S->bs) {
+        cudaFree(S->bs);
+        S->bs = nullptr;
+    }
 }
