@@ -5,7 +5,7 @@
 // Eq. blockiteration2, applied to the correction):
 //   r = b - A u          FP64 arithmetic, stored as FP32 (fused cast), ||r|| in FP64
 //   c = 0; m sweeps of the FP32 context on A c = r
-//   u = u + c            FP64 accumulate (and c is re-zeroed in the same pass)
+//   u = u + c            FP64 accumulate (and c re-zeroed in the same pass where it is read)
 // until ||r||_2 / ||b||_2 <= rtol.  Only the norm crosses to the host (one read per outer
 // step).
 #include <cmath>
@@ -15,12 +15,28 @@
 
 namespace {
 
-__global__ void correct_kernel(double* __restrict__ u, float* __restrict__ c, long long n)
+// u += c (n4 groups of four cells and the rest), and c = 0 where the next correction starts
+// from c.
+template <bool ZERO>
+__global__ void __launch_bounds__(256) correct_kernel(double* __restrict__ u, float* __restrict__ c,
+                                                      long long n)
 {
-    for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < n;
-         t += (long long)gridDim.x * blockDim.x) {
+    const long long n4 = n >> 2, stride = (long long)gridDim.x * blockDim.x;
+    const long long t0 = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    double2* u2 = reinterpret_cast<double2*>(u);
+    float4* c4 = reinterpret_cast<float4*>(c);
+    for (long long t = t0; t < n4; t += stride) {
+        const float4 d = c4[t];
+        double2 a = u2[2 * t], b = u2[2 * t + 1];
+        a.x += (double)d.x, a.y += (double)d.y, b.x += (double)d.z, b.y += (double)d.w;
+        u2[2 * t] = a, u2[2 * t + 1] = b;
+        if (ZERO)
+            c4[t] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    }
+    for (long long t = 4 * n4 + t0; t < n; t += stride) {
         u[t] += (double)c[t];
-        c[t] = 0.0f;
+        if (ZERO)
+            c[t] = 0.0f;
     }
 }
 
@@ -88,15 +104,22 @@ extern "C" int brsmooth_defect_correction(brs_ctx* outer, brs_ctx* inner, double
             history[it] = rel;
         if (rel <= rtol || it >= max_outer)
             break;
-        // c starts from zero: a plane context in the x-sine form skips c's transform
+        // c starts from zero: a plane context in the x-sine form skips c's transform (and never
+        // reads c)
+        bool reads_c = false;
         rc = inner->plane ? plane_modes_sweep(inner, inner->dc_c, inner->dc_r, inner_sweeps, s,
                                               true)
                           : BRS_ERR_UNSUPPORTED;
-        if (rc == BRS_ERR_UNSUPPORTED)
+        if (rc == BRS_ERR_UNSUPPORTED) {
+            reads_c = true;
             rc = brsmooth_sweep(inner, inner->dc_c, inner->dc_r, inner_sweeps, stream);
+        }
         if (rc != BRS_OK)
             return rc;
-        correct_kernel<<<blocks, 256, 0, s>>>(u, inner->dc_c, n);
+        if (reads_c)
+            correct_kernel<true><<<blocks, 256, 0, s>>>(u, inner->dc_c, n);
+        else
+            correct_kernel<false><<<blocks, 256, 0, s>>>(u, inner->dc_c, n);
         e = cudaGetLastError();
         if (e != cudaSuccess)
             return brs_cuda_status(e);

@@ -31,6 +31,14 @@ __device__ __forceinline__ void ld4(T (&v)[4], const T* p, int rem, bool vec)
 }
 
 template <typename T>
+__device__ __forceinline__ void zero4(T (&v)[4])
+{
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+        v[q] = T(0);
+}
+
+template <typename T>
 __device__ __forceinline__ void st4(T* p, const T (&v)[4], int rem, bool vec)
 {
     if (vec) {
@@ -52,7 +60,8 @@ __device__ __forceinline__ void st4(T* p, const T (&v)[4], int rem, bool vec)
 // grid, four cells per lane: no per-cell index division, and each CTA's partial sum of
 // squares covers a fixed set of cells.  Squares of an FP32 residual are summed in FP32 over
 // a lane's cells of one row and then in FP64 (the FP64 pipe is the narrow one on this part).
-template <typename T, typename TR>
+// NORM: r = b (the norm of b alone).
+template <typename T, typename TR, bool NORM>
 __global__ void __launch_bounds__(kResThreads) residual_kernel(const T* __restrict__ u,
                                                                const T* __restrict__ b,
                                                                TR* __restrict__ r, int nx, int ny,
@@ -74,45 +83,41 @@ __global__ void __launch_bounds__(kResThreads) residual_kernel(const T* __restri
             const int rem = nx - i0;
             const T* pu = u + base + i0;
             T uc[4], bv[4], a[4], c[4];
-            ld4(uc, pu, rem, vec);
+            if constexpr (!NORM)
+                ld4(uc, pu, rem, vec);
             ld4(bv, b + base + i0, rem, vec);
-            T sy[4], sz[4];
+            // neighbour sums; a row outside the grid is zeros (one addition per pair: FP64's cost
+            // here is its operations, 9 per cell with the cast)
+            T sy[4] = {}, sz[4] = {};
+            if constexpr (!NORM) {
+                T d[4] = {}, e[4] = {};
+                zero4(a), zero4(c);
+                if (j > 0)
+                    ld4(a, pu - nx, rem, vec);
+                if (j + 1 < ny)
+                    ld4(c, pu + nx, rem, vec);
+                if (k > 0)
+                    ld4(d, pu - plane, rem, vec);
+                if (k + 1 < nz)
+                    ld4(e, pu + plane, rem, vec);
 #pragma unroll
-            for (int q = 0; q < 4; ++q)
-                sy[q] = sz[q] = T(0);
-            if (j > 0) {
-                ld4(a, pu - nx, rem, vec);
-#pragma unroll
-                for (int q = 0; q < 4; ++q)
-                    sy[q] += a[q];
+                for (int q = 0; q < 4; ++q) {
+                    sy[q] = a[q] + c[q];
+                    sz[q] = d[q] + e[q];
+                }
             }
-            if (j + 1 < ny) {
-                ld4(c, pu + nx, rem, vec);
-#pragma unroll
-                for (int q = 0; q < 4; ++q)
-                    sy[q] += c[q];
-            }
-            if (k > 0) {
-                ld4(a, pu - plane, rem, vec);
-#pragma unroll
-                for (int q = 0; q < 4; ++q)
-                    sz[q] += a[q];
-            }
-            if (k + 1 < nz) {
-                ld4(c, pu + plane, rem, vec);
-#pragma unroll
-                for (int q = 0; q < 4; ++q)
-                    sz[q] += c[q];
-            }
-            const T left = i0 > 0 ? pu[-1] : T(0);
-            const T right = rem > 4 ? pu[4] : T(0);
+            const T left = !NORM && i0 > 0 ? pu[-1] : T(0);
+            const T right = !NORM && rem > 4 ? pu[4] : T(0);
             T rv[4];
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
                 const T l = q == 0 ? left : uc[q - 1];
                 const T rr = q == 3 ? right : (q + 1 < rem ? uc[q + 1] : T(0));
                 // b - A u = b - d u + ax sx + ay sy + az sz
-                rv[q] = fma(cz, sz[q], fma(cy, sy[q], fma(cx, l + rr, fma(-dg, uc[q], bv[q]))));
+                if constexpr (NORM)
+                    rv[q] = bv[q];
+                else
+                    rv[q] = fma(cz, sz[q], fma(cy, sy[q], fma(cx, l + rr, fma(-dg, uc[q], bv[q]))));
                 if (q < rem) {
                     if constexpr (sizeof(T) == 4)
                         sq = fma(rv[q], rv[q], sq);
@@ -182,7 +187,7 @@ int residual_setup(brs_ctx* c)
     return BRS_OK;
 }
 
-template <typename T, typename TR>
+template <typename T, typename TR, bool NORM = false>
 int residual_run(brs_ctx* c, const T* u, const T* b, TR* r, bool want_norm, double ax,
                  double ay, double az, cudaStream_t s)
 {
@@ -196,7 +201,7 @@ int residual_run(brs_ctx* c, const T* u, const T* b, TR* r, bool want_norm, doub
     double* part = want_norm ? c->partials : nullptr;
     auto a16 = [](const void* q) { return (reinterpret_cast<uintptr_t>(q) & 15u) == 0; };
     const bool vec = p.nx % 4 == 0 && a16(u) && a16(b) && (!r || a16(r));
-    residual_kernel<T, TR><<<blocks, kResThreads, 0, s>>>(u, b, r, p.nx, p.ny, p.nz, ax, ay, az,
+    residual_kernel<T, TR, NORM><<<blocks, kResThreads, 0, s>>>(u, b, r, p.nx, p.ny, p.nz, ax, ay, az,
                                                           part, vec);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess)
@@ -228,10 +233,9 @@ int residual_launch_f32out(brs_ctx* c, const double* u, const double* b, float* 
 
 int norm2sq_launch(brs_ctx* c, const void* x, cudaStream_t s)
 {
-    // with zero coefficients the residual kernel returns b itself: ||x||^2 into norm_dev
     if (c->p.dtype == BRS_F64)
-        return residual_run<double, double>(c, (const double*)x, (const double*)x, nullptr, true,
+        return residual_run<double, double, true>(c, (const double*)x, (const double*)x, nullptr, true,
                                             0.0, 0.0, 0.0, s);
-    return residual_run<float, float>(c, (const float*)x, (const float*)x, nullptr, true, 0.0,
-                                      0.0, 0.0, s);
+    return residual_run<float, float, true>(c, (const float*)x, (const float*)x, nullptr, true,
+                                            0.0, 0.0, 0.0, s);
 }
