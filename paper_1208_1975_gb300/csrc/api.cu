@@ -13,6 +13,7 @@
 #include "batched.cuh"
 #include "box.cuh"
 #include "line_tile.cuh"
+#include "line_two.cuh"
 #include "plane.cuh"
 
 namespace {
@@ -290,6 +291,8 @@ int brsmooth_create(const brs_params* p, brs_ctx** out)
     *c->dev_status = 0;
     if (p->block == BRS_XLINE) {
         rc = line_setup(c);
+        if (rc == BRS_OK)
+            rc = line_two_setup(c);
         // FP64 lines: the elimination from both ends (BRSMOOTH_LINE_SEQ=0: the lane-scan
         // kernel), on the caller's layout; grids with enough lines also hold the line-major
         // form for calls of several sweeps
@@ -370,8 +373,13 @@ int brsmooth_sweep(brs_ctx* c, void* u, const void* b, int nsweeps, void* stream
     // block Jacobi: v = u + omega M^{-1}(b - A u) into the second vector, then swap (Alg. 2)
     void* cur = u;
     void* nxt = c->scratch;
+    int pairs = line_two_pairs(c, nsweeps);
     for (int k = 0; k < nsweeps && rc == BRS_OK; ++k) {
-        rc = sweep_one(c, cur, nxt, b, s);
+        if (pairs > 0) {
+            rc = line_two_launch(c, cur, nxt, b, s);
+            --pairs, ++k;
+        } else
+            rc = sweep_one(c, cur, nxt, b, s);
         void* t = cur;
         cur = nxt;
         nxt = t;

@@ -57,6 +57,7 @@ struct brs_ctx {
     void* line_tab = nullptr;
     void* line_tab2 = nullptr;  // two-warp layout (LineCfg::pair), FP32
     LineCfg lcfg;
+    int two_stages = 0;         // ring stages of the two-sweep form (line_two.cu); 0: not taken
     // residual reduction
     double* partials = nullptr;
     int npartials = 0;

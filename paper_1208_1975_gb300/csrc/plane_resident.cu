@@ -26,7 +26,9 @@
 #include <type_traits>
 
 #include "line_impl.cuh"
+#include "line_many.cuh"
 #include "plane.cuh"
+#include "row_smem.cuh"
 #include "thomas_tables.h"
 
 namespace {
@@ -42,37 +44,7 @@ __device__ __forceinline__ void cluster_sync()
                  ::: "memory");
 }
 
-// Rows in shared memory: lane l's E cells start at l E, and for E = 8 its two 16-byte halves trade
-// places when l / 4 is odd, so that the 8 lanes of an access phase cover all banks.
-template <int E>
-__device__ __forceinline__ int cell_pos(int y)  // place of cell y in its row
-{
-    return E == 8 ? y ^ ((y >> 3) & 4) : y;
-}
-
-template <int E>
-__device__ __forceinline__ void ld_row(float (&v)[E], const float* row, int lane)
-{
-    const float4* p = reinterpret_cast<const float4*>(row + lane * E);
-    const int h = E == 8 ? (lane >> 2) & 1 : 0;
-#pragma unroll
-    for (int m = 0; m < E / 4; ++m) {
-        const float4 t = p[m ^ h];
-        v[4 * m] = t.x, v[4 * m + 1] = t.y, v[4 * m + 2] = t.z, v[4 * m + 3] = t.w;
-    }
-}
-
-template <int E>
-__device__ __forceinline__ void st_row(float* row, const float (&v)[E], int lane)
-{
-    float4* p = reinterpret_cast<float4*>(row + lane * E);
-    const int h = E == 8 ? (lane >> 2) & 1 : 0;
-#pragma unroll
-    for (int m = 0; m < E / 4; ++m)
-        p[m ^ h] = make_float4(v[4 * m], v[4 * m + 1], v[4 * m + 2], v[4 * m + 3]);
-}
-
-// ld_row from the same place in another CTA of the cluster.
+// row_ld from the same place in another CTA of the cluster.
 template <int E>
 __device__ __forceinline__ void ld_remote(float (&v)[E], const float* row, int rank, int lane)
 {
@@ -85,88 +57,6 @@ __device__ __forceinline__ void ld_remote(float (&v)[E], const float* row, int r
                      : "=f"(v[4 * m]), "=f"(v[4 * m + 1]), "=f"(v[4 * m + 2]), "=f"(v[4 * m + 3])
                      : "r"(a + 16 * (m ^ h))
                      : "memory");
-}
-
-// line_solve (line_impl.cuh) of M lines at once, step by step side by side: one line's chain of
-// multiply-adds and shuffles leaves most issue slots of its warp empty.
-template <int E, int G, int M>
-__device__ __forceinline__ void line_solve_many(float (&r)[M][E], const brs::LineTables<float, E, G>& tb,
-                                                int lane)
-{
-    constexpr int LG = brs::Log2<G>::value;
-    float z[M], B[M];
-#pragma unroll
-    for (int m = 0; m < M; ++m)
-        z[m] = 0.0f;
-#pragma unroll
-    for (int q = 0; q < E; ++q)
-#pragma unroll
-        for (int m = 0; m < M; ++m)
-            z[m] = fma(tb.c[q], z[m], r[m][q]);
-#pragma unroll
-    for (int m = 0; m < M; ++m)
-        B[m] = z[m];
-#pragma unroll
-    for (int t = 0; t < LG; ++t) {
-        const int d = 1 << t;
-        float Bp[M];
-#pragma unroll
-        for (int m = 0; m < M; ++m)
-            Bp[m] = __shfl_up_sync(0xffffffffu, B[m], d, G);
-#pragma unroll
-        for (int m = 0; m < M; ++m)
-            if (lane >= d)
-                B[m] = fma(tb.af[t], Bp[m], B[m]);
-    }
-#pragma unroll
-    for (int m = 0; m < M; ++m) {
-        z[m] = __shfl_up_sync(0xffffffffu, B[m], 1, G);
-        if (lane == 0)
-            z[m] = 0.0f;
-    }
-#pragma unroll
-    for (int q = 0; q < E; ++q)
-#pragma unroll
-        for (int m = 0; m < M; ++m) {
-            z[m] = fma(tb.c[q], z[m], r[m][q]);
-            r[m][q] = z[m];
-        }
-#pragma unroll
-    for (int m = 0; m < M; ++m)
-        z[m] = 0.0f;
-#pragma unroll
-    for (int q = E - 1; q >= 0; --q)
-#pragma unroll
-        for (int m = 0; m < M; ++m)
-            z[m] = fma(tb.e[q], z[m], r[m][q]);
-#pragma unroll
-    for (int m = 0; m < M; ++m)
-        B[m] = z[m];
-#pragma unroll
-    for (int t = 0; t < LG; ++t) {
-        const int d = 1 << t;
-        float Bn[M];
-#pragma unroll
-        for (int m = 0; m < M; ++m)
-            Bn[m] = __shfl_down_sync(0xffffffffu, B[m], d, G);
-#pragma unroll
-        for (int m = 0; m < M; ++m)
-            if (lane + d < G)
-                B[m] = fma(tb.ab[t], Bn[m], B[m]);
-    }
-#pragma unroll
-    for (int m = 0; m < M; ++m) {
-        z[m] = __shfl_down_sync(0xffffffffu, B[m], 1, G);
-        if (lane == G - 1)
-            z[m] = 0.0f;
-    }
-#pragma unroll
-    for (int q = E - 1; q >= 0; --q)
-#pragma unroll
-        for (int m = 0; m < M; ++m) {
-            z[m] = fma(tb.e[q], z[m], r[m][q]);
-            r[m][q] = z[m];
-        }
 }
 
 constexpr int res_threads(int E) { return E <= 8 ? 512 : 256; }
@@ -196,7 +86,7 @@ __global__ void __launch_bounds__(res_threads(E), 1) mode_resident_kernel(
     // row i of this CTA's planes; -1 and np are the neighbours' (zero outside the grid)
     auto row = [&](float (&v)[E], int i) {
         if (i >= 0 && i < np)
-            ld_row<E>(v, U + (size_t)i * NP, lane);
+            brs::row_ld<E>(v, U + (size_t)i * NP, lane);
         else if (i < 0 ? rank > 0 : rank + 1 < a.C)
             ld_remote<E>(v, U + (size_t)(i < 0 ? below : 0) * NP, i < 0 ? rank - 1 : rank + 1, lane);
         else
@@ -218,7 +108,7 @@ __global__ void __launch_bounds__(res_threads(E), 1) mode_resident_kernel(
                 const bool in = y < a.ny;
                 const float4 z = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
                 const long long o = base + i * pstride + y;
-                const int q = i * NP + cell_pos<E>(y);
+                const int q = i * NP + brs::row_pos<E>(y);
                 *reinterpret_cast<float4*>(U + q) = in ? *reinterpret_cast<const float4*>(u + o) : z;
                 *reinterpret_cast<float4*>(B + q) = in ? __ldg(reinterpret_cast<const float4*>(b + o)) : z;
             }
@@ -226,7 +116,7 @@ __global__ void __launch_bounds__(res_threads(E), 1) mode_resident_kernel(
             for (int t = threadIdx.x; t < np * NP; t += res_threads(E)) {
                 const int i = t / NP, y = t - i * NP;
                 const long long o = base + i * pstride + y;
-                const int q = i * NP + cell_pos<E>(y);
+                const int q = i * NP + brs::row_pos<E>(y);
                 U[q] = y < a.ny ? u[o] : 0.0f;
                 B[q] = y < a.ny ? __ldg(b + o) : 0.0f;
             }
@@ -268,7 +158,7 @@ __global__ void __launch_bounds__(res_threads(E), 1) mode_resident_kernel(
 #pragma unroll
                             for (int q = 0; q < E; ++q)
                                 up[q] = hi[q];
-                        ld_row<E>(bb, B + (size_t)ic * NP, lane);
+                        brs::row_ld<E>(bb, B + (size_t)ic * NP, lane);
 #pragma unroll
                         for (int q = 0; q < E; ++q)
                             r[m][q] = par ? fma(az, up[q], fma(az, um[q], bb[q]))
@@ -280,19 +170,19 @@ __global__ void __launch_bounds__(res_threads(E), 1) mode_resident_kernel(
                             for (int q = 0; q < E; ++q)
                                 um[q] = up[q];
                         } else
-                            ld_row<E>(um, U + (size_t)ic * NP, lane);
+                            brs::row_ld<E>(um, U + (size_t)ic * NP, lane);
                     }
-                    line_solve_many<E, G, M>(r, tb, lane);
+                    brs::line_solve_many<E, G, M>(r, tb, lane);
 #pragma unroll
                     for (int m = 0; m < M; ++m) {
                         float* own = U + (size_t)(i[m] < 0 ? 0 : i[m]) * NP;
                         float uc[E];
-                        ld_row<E>(uc, own, lane);
+                        brs::row_ld<E>(uc, own, lane);
 #pragma unroll
                         for (int q = 0; q < E; ++q)
                             r[m][q] = fma(tb.wp[q], r[m][q], om1 * uc[q]);
                         if (i[m] >= 0)
-                            st_row<E>(own, r[m], lane);
+                            brs::row_st<E>(own, r[m], lane);
                     }
                 };
                 int s = 0;
@@ -310,13 +200,13 @@ __global__ void __launch_bounds__(res_threads(E), 1) mode_resident_kernel(
                 const int i = t / n4, y = 4 * (t - i * n4);
                 if (y < a.ny)
                     *reinterpret_cast<float4*>(out + base + i * pstride + y) =
-                        *reinterpret_cast<const float4*>(U + i * NP + cell_pos<E>(y));
+                        *reinterpret_cast<const float4*>(U + i * NP + brs::row_pos<E>(y));
             }
         } else {
             for (int t = threadIdx.x; t < np * NP; t += res_threads(E)) {
                 const int i = t / NP, y = t - i * NP;
                 if (y < a.ny)
-                    out[base + i * pstride + y] = U[i * NP + cell_pos<E>(y)];
+                    out[base + i * pstride + y] = U[i * NP + brs::row_pos<E>(y)];
             }
         }
     }
