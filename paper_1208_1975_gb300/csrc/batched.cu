@@ -5,8 +5,8 @@
 // Work items are (patch, y-block of R lines, z-chunk of KC planes).  A persistent grid
 // of warps pulls items from an atomic counter (load balance across uneven patches);
 // each warp marches its R lines in +z: u(j,k-1), u(j,k), u(j,k+1) stay in registers,
-// the y neighbours inside the warp come by shuffle and only the two halo lines of the
-// y-block are loaded.  Lines are solved exactly with the shared-pivot Thomas scan of the
+// the y neighbours inside the warp come by shuffle (FP32 patches with aligned rows: from the
+// ring that stages them) and only the two halo lines of the y-block are loaded.  Lines are solved exactly with the shared-pivot Thomas scan of the
 // single-grid path (the factor of M_line depends only on nx and the coefficients, so one
 // table per distinct nx is built once).  One launch per sweep; the sweep sequence of a
 // call is captured once into a CUDA graph and replayed as a single graph launch.
@@ -52,6 +52,7 @@ struct BatchState {
     int KC = 8;                 // z-chunk
     int warps = 8;              // warps per CTA
     int grid = 0;               // persistent CTAs
+    int ctas_per_sm = 1;
     int nitems = 0;
     PatchDesc* d_desc = nullptr;
     int* d_item_patch = nullptr;
@@ -78,7 +79,7 @@ struct BatchState {
     bool keep = false;
     bool gvalid = false;
     int gpar = 0;
-    int stages = 4;             // its ring depth (z-steps of lookahead per warp)
+    int stages = 4;             // its ring depth (slots per warp)
 };
 
 BatchState* bs(brs_ctx* c)
@@ -87,16 +88,16 @@ BatchState* bs(brs_ctx* c)
 }
 
 constexpr int kE = 4;
-// cp.async ring fields: u(k+1), b(k) and the two halo lines
-constexpr int kFields = 4;
+// cp.async ring (FP32): a slot's rows of u (at most 96 16-byte pieces), then b
+constexpr int kSlotB = 96 * 16;
+constexpr int kSlotBytes = kSlotB + 32 * 16;
 // x ghosts of one work item of a level, staged per warp: 2 faces x z-steps x lines
 constexpr int kMaxKC = 32;
-constexpr size_t xg_bytes(size_t esize) { return (size_t)2 * kMaxKC * 8 * esize; }
-// bytes of one warp's cp.async area: stages x fields x 32 lanes x kE elements, plus the
-// staged x ghosts of a level
-constexpr size_t async_ring_bytes(int stages, size_t esize, bool level)
+constexpr size_t kXgBytes = (size_t)2 * kMaxKC * 8 * sizeof(float);
+// bytes of one warp's cp.async area: the ring, plus the staged x ghosts of a level
+constexpr size_t async_ring_bytes(int stages, bool level)
 {
-    return (size_t)stages * kFields * 32 * kE * esize + (level ? xg_bytes(esize) : 0);
+    return (size_t)stages * kSlotBytes + (level ? kXgBytes : 0);
 }
 
 // Ghost block of a patch of a level (the face neighbours' adjacent layers as they were before
@@ -367,21 +368,27 @@ __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commi
 template <int N>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
-// Same work item as batched_item, with the per-step inputs (u(k+1), b(k) and, for the
-// lines at the y-block edges, the halo lines j-1 / j+1 of plane k) staged by cp.async
-// through a per-warp ring of D steps in shared memory.  Every patch row is a
-// multiple of 16 bytes (checked on the host).  Each lane copies and reads back only its
-// own 16-byte pieces, so no cross-lane synchronisation is needed.
-template <typename T, int G, bool GS, int D, bool LV>
+// Same work item as batched_item in FP32, with the per-step inputs staged by cp.async through a
+// per-warp ring of D slots in shared memory.  The slot of step k holds b(k) of the warp's R lines
+// and plane k + 1 of u for them and one more line on each side, as R + 2 rows of G 16-byte pieces:
+// a lane's own piece, and those of the lines before and after it, lie G pieces apart.  Step k takes
+// u(k+1) and b(k) from its slot and the y neighbours from the slot before, which it then refills.
+// Every patch row is a multiple of 16 bytes (checked on the host).
+// Bound by the latency of a step's chain until enough warps are resident, then by DRAM: 600 patches
+// of 16 to 64 cells a side (38 M cells), us per sweep: with the y neighbours by shuffle and select,
+// and every row's address formed anew per step, 87 in 118 registers (16 warps per SM, 54 % of the
+// issue slots, DRAM 57 %); so, 82 with 16 warps and 76 with the 20 that 96 registers allow, 0.9 of
+// the copy rate.  24 warps in 80 registers: 78.
+template <int G, bool GS, int D, bool LV>
 __device__ __forceinline__ void batched_item_async(const PatchDesc& d, int jb, int kc, int KC,
-                                                   const T* uin, T* uout,
-                                                   const T* __restrict__ b,
-                                                   const T* __restrict__ tab, T ax, T ay, T az,
-                                                   T om1, const T* ghost, unsigned char* ring,
-                                                   T* gnext, const long long* pp)
+                                                   const float* uin, float* uout,
+                                                   const float* __restrict__ b,
+                                                   const float* __restrict__ tab, float ax,
+                                                   float ay, float az, float om1,
+                                                   const float* ghost, unsigned char* ring,
+                                                   float* gnext, const long long* pp)
 {
     constexpr int R = 32 / G;
-    constexpr int CH = (int)(kE * sizeof(T) / 16);  // 16-byte chunks per lane and field
     const int lanew = threadIdx.x & 31;
     const int g = lanew / G, l = lanew % G;
     const int nx = d.nx, ny = d.ny, nz = d.nz;
@@ -390,65 +397,62 @@ __device__ __forceinline__ void batched_item_async(const PatchDesc& d, int jb, i
     const int x0 = l * kE;
     const bool xin = x0 < nx;
     const long long plane = (long long)nx * ny;
-    const T* ub = uin + d.off;
-    T* uo = uout + d.off;
-    const T* bb = b + d.off;
-    brs::LineTables<T, kE, G> tb;
+    const float* ub = uin + d.off;
+    brs::LineTables<float, kE, G> tb;
     tb.load(tab + d.tab, l);
     const int k0 = kc * KC;
     const int k1 = min(nz, k0 + KC);
     const uint32_t ring0 = (uint32_t)__cvta_generic_to_shared(ring);
-    // byte offset of (slot, field, chunk) for this lane
-    auto soff = [&](int slot, int f, int c) -> uint32_t {
-        return (uint32_t)((((slot * kFields + f) * CH + c) * 32 + lanew) * 16);
+    // A row of u as the steps walk along z: its piece at x0 in the next plane, and the stride to
+    // the one after.  Rows outside the patch are the ghost rows of a level's y faces, or zero.
+    struct Row {
+        const float* p;
+        int step;
+        bool ok;
     };
-    // Rows of u this item may need from outside the patch (a level's ghost block, else
-    // none): row j of the z- and z+ faces, and the y- / y+ face rows of its edge lines.
-    const T* gzm = nullptr;
-    const T* gzp = nullptr;
-    const T* gym = nullptr;
-    const T* gyp = nullptr;
-    if (LV) {
-        gzm = outside_row(d, ghost, j, -1);
-        gzp = outside_row(d, ghost, j, nz);
-        gym = outside_row(d, ghost, -1, 0);   // + kk * nx for plane kk
-        gyp = outside_row(d, ghost, ny, 0);
-    }
-    // row (jj, kk) of src: inside the patch, else the ghost row (u of a level), else zeros
-    auto row_of = [&](const T* src, int jj, int kk) -> const T* {
-        if (jj >= 0 && jj < ny && kk >= 0 && kk < nz)
-            return src + (long long)kk * plane + (long long)jj * nx;
-        if (!LV || src != ub)
-            return nullptr;
-        if (kk == -1)
-            return jj == j ? gzm : nullptr;
-        if (kk == nz)
-            return jj == j ? gzp : nullptr;
-        if (jj == -1)
-            return gym ? gym + (long long)kk * nx : nullptr;
-        if (jj == ny)
-            return gyp ? gyp + (long long)kk * nx : nullptr;
-        return nullptr;
+    auto row_at = [&](int jj) -> Row {
+        Row r{ub, 0, false};
+        if (jj >= 0 && jj < ny)
+            r = {ub + (long long)k0 * plane + (long long)jj * nx + x0, nx * ny, xin};
+        else if (LV && (jj == -1 || jj == ny)) {
+            const float* gy = outside_row(d, ghost, jj, 0);
+            if (gy)
+                r = {gy + (long long)k0 * nx + x0, nx, xin};
+        }
+        return r;
     };
-    // The steps' rows are issued for consecutive planes k0, k0 + 1, ...: their element
-    // offsets advance by one plane (a y face's ghost rows by nx) per step, and whether
-    // each field's row exists is fixed per item.  (The generic selection of row_of on
-    // every copy cost about a fifth of the kernel's instructions.)
-    long long o_next = (long long)k0 * plane + (long long)j * nx + x0;  // row (j, k) at x0
+    Row own = row_at(j);
+    // the lines before and after the warp's: lanes 0 .. G-1 and G .. 2G-1 (G = 32: both)
+    Row edge = row_at(G == 32 || lanew < G ? jb * R - 1 : lanew < 2 * G ? jb * R + R : -2);
+    Row edge2 = row_at(G == 32 ? jb * R + R : -2);
+    const uint32_t edge_at = (uint32_t)((G == 32 || lanew < G ? lanew : 32 + lanew) * 16);
+    const float* pb = b + d.off + (long long)k0 * plane + (long long)j * nx + x0;
     const bool ok_b = xin && jin;
-    const bool ok_n = xin && j >= 1 && j <= ny;  // line j - 1 inside the patch
-    const bool ok_s = xin && j + 1 < ny;         // line j + 1
-    // a level's rows outside the patch: u(k+1) of line ny is the y+ ghost row, and the
-    // halo lines at the patch's y faces are the y- / y+ ghost rows
-    long long og_next = (long long)k0 * nx + x0;
-    const bool ok_0 = xin && (jin || (j == ny && gyp));
-    const bool ok_gn = xin && (j > 0 || gym);
-    const bool ok_gs = xin && (j + 1 < ny || (j + 1 == ny && gyp));
-    auto copy_at = [&](int slot, int f, const T* src, long long o, bool ok) {
-        const T* p = ok ? src + o : ub;
-#pragma unroll
-        for (int c = 0; c < CH; ++c)
-            cp_async16(ring0 + soff(slot, f, c), p + c * (16 / sizeof(T)), ok ? 16u : 0u);
+    const float* gzp = LV && jin ? outside_row(d, ghost, j, nz) : nullptr;
+    auto copy = [&](uint32_t dst, const Row& r) {
+        cp_async16(dst, r.ok ? r.p : ub, r.ok ? 16u : 0u);
+    };
+    // plane kk of u and, unless first, b(kk - 1)
+    auto issue = [&](int kk, uint32_t slot, bool first) {
+        if (kk == nz) {
+            own.p = LV && gzp ? gzp + x0 : ub;
+            own.ok = LV && gzp && xin;
+        }
+        copy(slot + (uint32_t)(lanew + G) * 16, own);
+        own.p += own.step;
+        if (kk < nz) {  // the y neighbours of plane nz are not used
+            if (G == 32 || lanew < 2 * G)
+                copy(slot + edge_at, edge);
+            edge.p += edge.step;
+            if constexpr (G == 32) {
+                copy(slot + (uint32_t)(lanew + 2 * G) * 16, edge2);
+                edge2.p += edge2.step;
+            }
+        }
+        if (!first) {
+            cp_async16(slot + kSlotB + lanew * 16, ok_b ? pb : ub, ok_b ? 16u : 0u);
+            pb += plane;
+        }
     };
     // x ghosts of the line (level contexts): the lanes holding x = 0 and x = nx - 1
     const bool xlo = LV && xin && jin && x0 == 0;
@@ -464,112 +468,73 @@ __device__ __forceinline__ void batched_item_async(const PatchDesc& d, int jb, i
             gy = o + (long long)k0 * nx + x0;
     }
     // the item's x ghosts, staged once: xg[face][k - k0][line in the warp], copied
-    // asynchronously with the first step's inputs (zero beyond the last line)
-    T* xg = reinterpret_cast<T*>(ring + (size_t)D * kFields * 32 * kE * sizeof(T));
+    // asynchronously with the first plane (zero beyond the last line)
+    float* xg = reinterpret_cast<float*>(ring + (size_t)D * kSlotBytes);
     if (LV) {
         // x faces are [k][j] in the ghost block: element (kk, jl) of the item at
         // xb + face * xpo + kk * ny + jl (R a power of two: no divisions)
         const long long xpo = round4((long long)ny * nz);
         const int nk = k1 - k0;
         const uint32_t xg0 = (uint32_t)__cvta_generic_to_shared(xg);
-        const T* xb = ghost_x(d, ghost, jb * R, k0);
+        const float* xb = ghost_x(d, ghost, jb * R, k0);
         for (int face = 0; face < 2; ++face)
             for (int idx = lanew; idx < nk * R; idx += 32) {
                 const int kk = idx / R, jl = idx % R;
                 const bool ok = jb * R + jl < ny;
-                const T* src = ok ? xb + (face ? xpo : 0) + (long long)kk * ny + jl : ghost;
-                cp_async4(xg0 + (uint32_t)(((face * kMaxKC + kk) * 8 + jl) * sizeof(T)), src,
+                const float* src = ok ? xb + (face ? xpo : 0) + (long long)kk * ny + jl : ghost;
+                cp_async4(xg0 + (uint32_t)(((face * kMaxKC + kk) * 8 + jl) * sizeof(float)), src,
                           ok ? 4u : 0u);
             }
     }
-    auto issue = [&](int kk, int slot) {
-        if constexpr (LV) {
-            // the rows this step can need outside the patch are known per field: u(k+1)
-            // crosses the z+ face on the last plane, the halo lines cross the y faces, and
-            // line ny (past the patch, in the last y-block) carries the y+ ghost row that
-            // its neighbour ny - 1 takes by shuffle (og: row kk of a y face, at x0)
-            const long long o = o_next, og = og_next;
-            o_next += plane;
-            og_next += nx;
-            if (kk + 1 < nz)
-                copy_at(slot, 0, jin ? ub : gyp, jin ? o + plane : og + nx, ok_0);
-            else
-                copy_at(slot, 0, gzp, x0, xin && gzp);
-            copy_at(slot, 1, bb, o, ok_b);
-            if (g == 0)
-                copy_at(slot, 2, j > 0 ? ub : gym, j > 0 ? o - nx : og, ok_gn);
-            if (g == R - 1)
-                copy_at(slot, 3, j + 1 < ny ? ub : gyp, j + 1 < ny ? o + nx : og, ok_gs);
-        } else {
-            const long long o = o_next;  // row (j, kk): issue runs for kk = k0, k0 + 1, ...
-            o_next += plane;
-            copy_at(slot, 0, ub, o + plane, ok_b && kk + 1 < nz);
-            copy_at(slot, 1, bb, o, ok_b);
-            if (g == 0)
-                copy_at(slot, 2, ub, o - nx, ok_n);
-            if (g == R - 1)
-                copy_at(slot, 3, ub, o + nx, ok_s);
-        }
+    auto ld4 = [](float (&v)[kE], const float* p) {
+        *reinterpret_cast<float4*>(v) = *reinterpret_cast<const float4*>(p);
     };
-    auto read = [&](int slot, int f, T (&v)[kE]) {
-#pragma unroll
-        for (int c = 0; c < CH; ++c)
-            reinterpret_cast<float4*>(v)[c] =
-                *reinterpret_cast<const float4*>(ring + soff(slot, f, c));
-    };
-    auto ld = [&](const T* src, int jj, int kk, T (&v)[kE]) {
-        const T* row = row_of(src, jj, kk);
-        if (xin && row) {
-            const T* p = row + x0;
-#pragma unroll
-            for (int c = 0; c < CH; ++c)
-                reinterpret_cast<float4*>(v)[c] = reinterpret_cast<const float4*>(p)[c];
-        } else {
-#pragma unroll
-            for (int q = 0; q < kE; ++q)
-                v[q] = T(0);
-        }
-    };
+    const float* mine = reinterpret_cast<const float*>(ring) + lanew * kE;  // in slot 0
+    constexpr int SW = kSlotBytes / 4;
 
-    T um[kE], uc[kE], up[kE], r[kE], bv[kE], un[kE], us[kE], hn[kE], hs[kE];
-    ld(ub, j, k0 - 1, um);
-    ld(ub, j, k0, uc);
+    float um[kE] = {0.0f, 0.0f, 0.0f, 0.0f}, uc[kE], up[kE], r[kE], bv[kE], un[kE], us[kE];
+    if (ok_b) {
+        const float* pm = k0 > 0 ? ub + (long long)(k0 - 1) * plane + (long long)j * nx
+                                 : LV ? outside_row(d, ghost, j, -1) : nullptr;
+        if (pm)
+            ld4(um, pm + x0);
+    }
 #pragma unroll
     for (int i = 0; i < D; ++i) {
-        if (k0 + i < k1)
-            issue(k0 + i, i);
+        if (k0 + i <= k1)
+            issue(k0 + i, ring0 + i * kSlotBytes, i == 0);
         cp_async_commit();
     }
-    if (LV) {  // the x ghosts (first group) have landed and every lane sees them
-        cp_async_wait<D - 1>();
-        __syncwarp();
-    }
-    int slot = 0;
+    cp_async_wait<D - 1>();
+    __syncwarp();  // plane k0 and the x ghosts have landed and every lane sees them
+    ld4(uc, mine + G * kE);
+    int prv = 0, cur = 1;  // slots of step k - 1 (plane k) and step k
+    float* po = uout + d.off + (long long)k0 * plane + (long long)j * nx + x0;
     for (int k = k0; k < k1; ++k) {
-        cp_async_wait<D - 1>();  // the group of step k (committed D groups ago) is complete
-        read(slot, 0, up);
-        read(slot, 1, bv);
-        if (g == 0)
-            read(slot, 2, hn);
-        if (g == R - 1)
-            read(slot, 3, hs);
-        T gxm = T(0), gxp = T(0);
+        cp_async_wait<D - 2>();  // the group of step k is complete
+        __syncwarp();
+        const float *sp = mine + prv * SW, *sc = mine + cur * SW;
+        ld4(un, sp);
+        ld4(us, sp + 2 * G * kE);
+        ld4(up, sc + G * kE);
+        ld4(bv, sc + kSlotB / 4);
+        float gxm = 0.0f, gxp = 0.0f;
         if (LV) {
             if (xlo)
                 gxm = xg[(k - k0) * 8 + g];
             if (xhi)
                 gxp = xg[(kMaxKC + k - k0) * 8 + g];
         }
-#pragma unroll
-        for (int q = 0; q < kE; ++q) {
-            T a = __shfl_up_sync(0xffffffffu, uc[q], G);
-            T c = __shfl_down_sync(0xffffffffu, uc[q], G);
-            un[q] = (g == 0) ? hn[q] : a;
-            us[q] = (g == R - 1) ? hs[q] : c;
-        }
+        __syncwarp();  // every lane has read the slot before: refill it
+        if (k + D <= k1)
+            issue(k + D, ring0 + prv * kSlotBytes, false);
+        cp_async_commit();
+        prv = cur;
+        cur = cur + 1 == D ? 0 : cur + 1;
+        // zero beyond the row; lines beyond the patch compute values that nothing reads
 #pragma unroll
         for (int q = 0; q < kE; ++q)
-            r[q] = (xin && jin) ? fma(az, um[q] + up[q], fma(ay, un[q] + us[q], bv[q])) : T(0);
+            r[q] = fma(az, um[q] + up[q], fma(ay, un[q] + us[q], bv[q]));
         if (xlo)
             r[0] = fma(ax, gxm, r[0]);
         if (xhi) {
@@ -578,70 +543,58 @@ __device__ __forceinline__ void batched_item_async(const PatchDesc& d, int jb, i
                 if (x0 + q == nx - 1)
                     r[q] = fma(ax, gxp, r[q]);
         }
-        brs::line_solve<T, kE, G>(r, tb, l);
-        T v[kE];
+        brs::line_solve<float, kE, G>(r, tb, l);
+        float v[kE];
 #pragma unroll
         for (int q = 0; q < kE; ++q)
             v[q] = fma(tb.wp[q], r[q], om1 * uc[q]);
-        if (xin && jin) {
-            T* p = uo + (long long)k * plane + (long long)j * nx + x0;
-#pragma unroll
-            for (int c = 0; c < CH; ++c)
-                reinterpret_cast<float4*>(p)[c] = reinterpret_cast<const float4*>(v)[c];
-        }
+        if (ok_b)
+            *reinterpret_cast<float4*>(po) = *reinterpret_cast<const float4*>(v);
+        po += plane;
         if constexpr (LV) {
             if (gy >= 0) {
-#pragma unroll
-                for (int c = 0; c < CH; ++c)
-                    reinterpret_cast<float4*>(gnext + gy)[c] = reinterpret_cast<const float4*>(v)[c];
+                *reinterpret_cast<float4*>(gnext + gy) = *reinterpret_cast<const float4*>(v);
                 gy += nx;
             }
             if (gnext && (k == 0 || k == nz - 1) && xin && jin) {  // k is the same for the warp
 #pragma unroll
                 for (int f = 4; f < 6; ++f) {
                     const long long o = (f == 4 ? k == 0 : k == nz - 1) ? __ldg(pp + f) : -1;
-                    if (o >= 0) {
-                        T* p = gnext + o + (long long)j * nx + x0;
-#pragma unroll
-                        for (int c = 0; c < CH; ++c)
-                            reinterpret_cast<float4*>(p)[c] = reinterpret_cast<const float4*>(v)[c];
-                    }
+                    if (o >= 0)
+                        *reinterpret_cast<float4*>(gnext + o + (long long)j * nx + x0) =
+                            *reinterpret_cast<const float4*>(v);
                 }
             }
         }
-
 #pragma unroll
         for (int q = 0; q < kE; ++q) {
-            um[q] = GS ? ((xin && jin) ? v[q] : T(0)) : uc[q];
+            um[q] = GS ? (ok_b ? v[q] : 0.0f) : uc[q];
             uc[q] = up[q];
         }
-        // refill the slot just read (its values have been consumed above)
-        if (k + D < k1)
-            issue(k + D, slot);
-        cp_async_commit();
-        slot = slot + 1 == D ? 0 : slot + 1;
     }
-    cp_async_wait<0>();  // only empty groups remain; the ring is free for the next item
-    __syncwarp();        // and every lane has read the staged x ghosts
+    cp_async_wait<0>();  // only empty groups remain
+    __syncwarp();        // and every lane has read its last slot and ghosts: the ring is free
 }
 
-template <typename T, bool GS, int D, bool LV>
-__global__ void __launch_bounds__(512) batched_async_kernel(const PatchDesc* __restrict__ desc,
+constexpr int kAsyncThreads = 256;
+
+template <bool GS, int D, bool LV>
+__global__ void __launch_bounds__(kAsyncThreads, 2) batched_async_kernel(const PatchDesc* __restrict__ desc,
                                                             const int* __restrict__ item_patch,
                                                             int nitems, int* counter, int KC,
-                                                            const T* uin, T* uout,
-                                                            const T* __restrict__ b,
-                                                            const T* __restrict__ tab,
+                                                            const float* uin, float* uout,
+                                                            const float* __restrict__ b,
+                                                            const float* __restrict__ tab,
                                                             double ax, double ay, double az,
-                                                            double om1, const T* ghost,
-                                                            T* gnext,
+                                                            double om1, const float* ghost,
+                                                            float* gnext,
                                                             const long long* __restrict__ push)
 {
     extern __shared__ __align__(16) unsigned char async_smem[];
     pdl_wait_trigger();
     const int lanew = threadIdx.x & 31;
     unsigned char* ring =
-        async_smem + (size_t)(threadIdx.x >> 5) * async_ring_bytes(D, sizeof(T), LV);
+        async_smem + (size_t)(threadIdx.x >> 5) * async_ring_bytes(D, LV);
     while (true) {
         int item = 0;
         if (lanew == 0)
@@ -655,13 +608,13 @@ __global__ void __launch_bounds__(512) batched_async_kernel(const PatchDesc* __r
         const int jb = local % d.njb, kc = local / d.njb;
         const long long* pp = push ? push + 6 * pq : nullptr;
         switch (d.cls) {
-        case 0: batched_item_async<T, 4, GS, D, LV>(d, jb, kc, KC, uin, uout, b, tab, (T)ax, (T)ay, (T)az, (T)om1, ghost, ring, gnext, pp); break;
-        case 1: batched_item_async<T, 8, GS, D, LV>(d, jb, kc, KC, uin, uout, b, tab, (T)ax, (T)ay, (T)az, (T)om1, ghost, ring, gnext, pp); break;
-        case 2: batched_item_async<T, 16, GS, D, LV>(d, jb, kc, KC, uin, uout, b, tab, (T)ax, (T)ay, (T)az, (T)om1, ghost, ring, gnext, pp); break;
-        default: batched_item_async<T, 32, GS, D, LV>(d, jb, kc, KC, uin, uout, b, tab, (T)ax, (T)ay, (T)az, (T)om1, ghost, ring, gnext, pp); break;
+        case 0: batched_item_async<4, GS, D, LV>(d, jb, kc, KC, uin, uout, b, tab, (float)ax, (float)ay, (float)az, (float)om1, ghost, ring, gnext, pp); break;
+        case 1: batched_item_async<8, GS, D, LV>(d, jb, kc, KC, uin, uout, b, tab, (float)ax, (float)ay, (float)az, (float)om1, ghost, ring, gnext, pp); break;
+        case 2: batched_item_async<16, GS, D, LV>(d, jb, kc, KC, uin, uout, b, tab, (float)ax, (float)ay, (float)az, (float)om1, ghost, ring, gnext, pp); break;
+        default: batched_item_async<32, GS, D, LV>(d, jb, kc, KC, uin, uout, b, tab, (float)ax, (float)ay, (float)az, (float)om1, ghost, ring, gnext, pp); break;
         }
         if (LV && gnext)
-            push_item<T>(desc, push, gnext, uout, item_patch[item], item, KC, true);
+            push_item<float>(desc, push, gnext, uout, item_patch[item], item, KC, true);
     }
 }
 
@@ -764,13 +717,13 @@ template <bool LV>
 const void* async_kernel_lv(bool gs, int stages)
 {
     if (stages >= 8)
-        return gs ? (const void*)batched_async_kernel<float, true, 8, LV>
-                  : (const void*)batched_async_kernel<float, false, 8, LV>;
+        return gs ? (const void*)batched_async_kernel<true, 8, LV>
+                  : (const void*)batched_async_kernel<false, 8, LV>;
     if (stages >= 6)
-        return gs ? (const void*)batched_async_kernel<float, true, 6, LV>
-                  : (const void*)batched_async_kernel<float, false, 6, LV>;
-    return gs ? (const void*)batched_async_kernel<float, true, 4, LV>
-              : (const void*)batched_async_kernel<float, false, 4, LV>;
+        return gs ? (const void*)batched_async_kernel<true, 6, LV>
+                  : (const void*)batched_async_kernel<false, 6, LV>;
+    return gs ? (const void*)batched_async_kernel<true, 4, LV>
+              : (const void*)batched_async_kernel<false, 4, LV>;
 }
 
 const void* async_kernel_for(bool gs, int stages, bool level)
@@ -859,7 +812,7 @@ int launch_one(brs_ctx* c, const void* uin, void* uout, const void* b, int* coun
     const void* k = B->async ? async_kernel_for(gs, B->stages, B->level)
                              : kernel_for(c->p.dtype, gs, B->level);
     const size_t smem =
-        B->async ? (size_t)B->warps * async_ring_bytes(B->stages, c->esize, B->level) : 0;
+        B->async ? (size_t)B->warps * async_ring_bytes(B->stages, B->level) : 0;
     const PatchDesc* desc = B->d_desc;
     const int* ip = B->d_item_patch;
     int nitems = B->nitems, KC = B->KC;
@@ -935,12 +888,19 @@ int env_int(const char* name, int dflt)
     return (v && *v) ? std::atoi(v) : dflt;
 }
 
+// The cp.async rings of every resident warp fit one SM.
+bool async_fits(const BatchState* B, int warps, int ctas_per_sm, bool level)
+{
+    return (size_t)warps * ctas_per_sm * async_ring_bytes(B->stages, level) <= 220u * 1024u;
+}
+
 void set_shape(brs_ctx* c, int warps, int ctas_per_sm)
 {
     BatchState* B = bs(c);
     int sms = 0;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
     B->warps = warps;
+    B->ctas_per_sm = ctas_per_sm;
     B->grid = std::max(1, sms * ctas_per_sm);
 }
 
@@ -980,13 +940,13 @@ int autotune(brs_ctx* c)
     std::vector<TuneVal> cands;
     for (int kc : {4, 8, 16, 32})
         for (int w : {4, 8, 16})
-            for (int cps : {2, 4, 8}) {
-                if (w * cps > 64)
+            for (int cps : {2, 4, 5, 8}) {
+                if (w * cps > 64 || (!B->async && cps == 5))
                     continue;
-                if (B->async &&
-                    ((size_t)w * cps * async_ring_bytes(B->stages, c->esize, true) > 220u * 1024u ||
-                     (size_t)w * async_ring_bytes(B->stages, c->esize, true) > 227u * 1024u))
-                    continue;  // the rings of every resident warp must fit one SM
+                // cp.async kernel: 8 or 20 warps per SM in CTAs of 4 warps, 16 in CTAs of 8
+                if (B->async && (w * 32 > kAsyncThreads || cps == 4 ||
+                                 !async_fits(B, w, cps, false)))
+                    continue;
                 if (fixed_kc && kc != fixed_kc)
                     continue;
                 cands.push_back({kc, w, cps});
@@ -1018,9 +978,10 @@ int autotune(brs_ctx* c)
         if (rc != BRS_OK)
             break;
         rc = enqueue_sweeps(c, tu, tb, 1, nullptr);  // warm
-        // best of two 5-sweep timings: one short timing picked shapes 8 % apart run to run
+        // best of two 5-sweep timings: one short timing picked shapes 8 % apart run to run (four of
+        // sweeps under 12 us, where launches scatter)
         float ms = 1e30f;
-        for (int rep = 0; rep < 2 && rc == BRS_OK; ++rep) {
+        for (int rep = 0; rep < (ms < 0.06f ? 4 : 2) && rc == BRS_OK; ++rep) {
             cudaEventRecord(e0, nullptr);
             rc = enqueue_sweeps(c, tu, tb, 5, nullptr);
             cudaEventRecord(e1, nullptr);
@@ -1030,7 +991,8 @@ int autotune(brs_ctx* c)
             cudaEventElapsedTime(&t, e0, e1);
             ms = t < ms ? t : ms;
         }
-        if (rc == BRS_OK && ms < best_ms) {
+        // fewer warps where more gain nothing
+        if (rc == BRS_OK && ms < 0.98f * best_ms) {
             best_ms = ms;
             best = v;
         }
@@ -1119,7 +1081,7 @@ int batched_setup(brs_ctx* c, int npatch, const int* dims)
         // both the plain and the level kernel (a level is set up after the tuner ran)
         for (bool lv : {false, true}) {
             const size_t want =
-                std::min<size_t>(227u * 1024u, 16 * async_ring_bytes(B->stages, c->esize, lv));
+                std::min<size_t>(227u * 1024u, 16 * async_ring_bytes(B->stages, lv));
             const void* k = async_kernel_for(c->p.method == BRS_CHAOTIC_GS, B->stages, lv);
             cudaFuncAttributes fa{};
             e = cudaFuncGetAttributes(&fa, k);
@@ -1143,6 +1105,11 @@ int level_setup(brs_ctx* c, const int* nbr)
 {
     BatchState* B = bs(c);
     B->level = true;
+    // a level's rings also hold its x ghosts, and its kernel has more registers
+    while (B->async && B->ctas_per_sm > 1 &&
+           (B->warps * B->ctas_per_sm > 16 ||
+            !async_fits(B, B->warps, B->ctas_per_sm, true)))
+        set_shape(c, B->warps, B->ctas_per_sm - 1);
     // boundary-cell chunks per patch (every dim >= 2, checked by the caller)
     std::vector<int> chunk_patch;
     long long gtotal = 0;
