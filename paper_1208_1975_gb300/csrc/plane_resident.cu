@@ -15,12 +15,16 @@
 // cluster barriers per sweep order all of it.  The operations on a cell are those of
 // mode_tma_kernel, in its order, so the results are the same bit for bit.  Rows are padded to
 // G E cells with zeros (zero table entries keep them zero), so any ny up to 512 does.
-// Bound by instruction issue: about 165 warp instructions per 256-cell line, and a phase of two
-// lines per warp takes 2000 clocks (0.65 of the issue rate); two lines are solved side by side,
-// because one line's chain leaves most of its warp's issue slots empty (24 -> 20 us per sweep).
-// us per sweep at 256^3, same box, streaming -> here: Jacobi 34.4 -> 20.2, Gauss-Seidel 47 -> 20.7;
-// 128^3 10.3 / 13.2 -> 2.6; 200x190x180, which had no streaming form and ran two transforms per
-// sweep, calls of 50 17.0 / 18.8 ms -> 0.99.
+// Bound by the latency of a phase, two lines per warp and a cluster barrier: 40 % of the issue
+// slots, most stalls on shared memory and the scans' shuffles.  Two lines are solved side by side,
+// because one line's chain leaves most of its warp's issue slots empty (24 -> 20.7 us per sweep).
+// Where a line takes the whole warp, a warp's share of the planes is warp-uniform and it steps
+// through exactly its own lines: no masked lines, one row pointer, 137 warp instructions per
+// 256-cell line instead of 165 (20.7 -> 18.5 us).  256-cell lines on 16 lanes of 16 cells, with a
+// sixth fewer instructions, gained nothing here (Gauss-Seidel 20.9).
+// us per sweep at 256^3, same box, streaming -> here: Jacobi 34.4 -> 18.5, Gauss-Seidel 47 -> 18.5;
+// 128^3 10.3 / 13.2 -> 2.1 / 2.3; 200x190x180, which had no streaming form and ran two transforms
+// per sweep, calls of 50 17.0 / 18.8 ms -> 0.81 / 0.86.
 #include <algorithm>
 #include <cstdlib>
 #include <type_traits>
@@ -74,7 +78,9 @@ __global__ void __launch_bounds__(res_threads(E), 1) mode_resident_kernel(
     auto first = [&](int r) { return (int)((long long)r * a.nz / a.C); };
     const int ks = first(rank), np = first(rank + 1) - ks;
     const int below = rank > 0 ? ks - first(rank - 1) - 1 : 0;  // the lower CTA's last row
-    const int g = threadIdx.x / G, lane = threadIdx.x % G;
+    // G = 32: the group is the warp, and so is its share of the planes
+    const int g = G == 32 ? __shfl_sync(0xffffffffu, threadIdx.x / 32, 0) : threadIdx.x / G;
+    const int lane = threadIdx.x % G;
     const float az = a.az, om1 = a.om1;
     const long long pstride = (long long)a.nm * a.ny;
     auto sync = [&]() {
@@ -122,77 +128,93 @@ __global__ void __launch_bounds__(res_threads(E), 1) mode_resident_kernel(
             }
         }
         sync();
-        for (int it = 0; it < a.nsweeps; ++it) {
-            // phases: Jacobi one (planes i, i + 1, ...), Gauss-Seidel two (planes of one parity)
-            constexpr int ST = GS ? 2 : 1;
-#pragma unroll 1
-            for (int par = 0; par < ST; ++par) {
-                const int f = GS ? (ks + par) & 1 : 0;     // first own plane of the phase
-                const int cnt = (np - f + ST - 1) / ST;    // how many
-                const int j0 = g * cnt / NG, j1 = (g + 1) * cnt / NG;
-                const int most = (cnt + NG - 1) / NG;
-                // um: the plane before the step's first one (Jacobi: its old values); hi: Jacobi's
-                // old plane after the run
-                float um[E], hi[E];
-                row(um, j0 < j1 ? f + ST * j0 - 1 : 0);
-                if constexpr (!GS) {
-                    row(hi, j1);
-                    sync();
-                }
-                // M lines of every group from its s-th on
-                auto step = [&](auto many, int s) {
-                    constexpr int M = decltype(many)::value;
-                    if (!__any_sync(0xffffffffu, j0 + s < j1))
-                        return;  // none in this warp
-                    float r[M][E];
-                    int i[M];
-#pragma unroll
-                    for (int m = 0; m < M; ++m) {
-                        const int j = j0 + s + m;
-                        i[m] = j < j1 ? f + ST * j : -1;
-                        const int ic = i[m] < 0 ? 0 : i[m];
-                        float up[E], bb[E];
-                        if (GS || j + 1 < j1)
-                            row(up, i[m] < 0 ? 0 : ic + 1);
-                        else
-#pragma unroll
-                            for (int q = 0; q < E; ++q)
-                                up[q] = hi[q];
-                        brs::row_ld<E>(bb, B + (size_t)ic * NP, lane);
-#pragma unroll
-                        for (int q = 0; q < E; ++q)
-                            r[m][q] = par ? fma(az, up[q], fma(az, um[q], bb[q]))
-                                          : fma(az, um[q] + up[q], bb[q]);
-                        // the next line's lower neighbour: its old own row (Jacobi), or the row
-                        // above this line (the other parity)
-                        if constexpr (GS) {
-#pragma unroll
-                            for (int q = 0; q < E; ++q)
-                                um[q] = up[q];
-                        } else
-                            brs::row_ld<E>(um, U + (size_t)ic * NP, lane);
-                    }
-                    brs::line_solve_many<E, G, M>(r, tb, lane);
-#pragma unroll
-                    for (int m = 0; m < M; ++m) {
-                        float* own = U + (size_t)(i[m] < 0 ? 0 : i[m]) * NP;
-                        float uc[E];
-                        brs::row_ld<E>(uc, own, lane);
-#pragma unroll
-                        for (int q = 0; q < E; ++q)
-                            r[m][q] = fma(tb.wp[q], r[m][q], om1 * uc[q]);
-                        if (i[m] >= 0)
-                            brs::row_st<E>(own, r[m], lane);
-                    }
-                };
-                int s = 0;
-#pragma unroll 1
-                for (; s + 1 < most; s += 2)
-                    step(std::integral_constant<int, 2>(), s);
-                if (s < most)
-                    step(std::integral_constant<int, 1>(), s);
+        // one phase: Jacobi all planes, Gauss-Seidel those of one parity
+        auto phase = [&](auto parity) {
+            constexpr int PAR = decltype(parity)::value, ST = GS ? 2 : 1;
+            const int f = GS ? (ks + PAR) & 1 : 0;     // first own plane of the phase
+            const int cnt = (np - f + ST - 1) / ST;    // how many
+            const int j0 = g * cnt / NG, j1 = (g + 1) * cnt / NG, n = j1 - j0;
+            // um: the plane before the next line (Jacobi: its old values); hi: the one after the run
+            float um[E], hi[E];
+            const int i0 = n > 0 ? f + ST * j0 : 0;  // groups without a line look at row 0
+            row(um, n > 0 ? i0 - 1 : 0);
+            row(hi, n > 0 ? f + ST * (j1 - 1) + 1 : 0);
+            if constexpr (!GS)
                 sync();
+            float* own = U + (size_t)i0 * NP;
+            const float* brow = B + (size_t)i0 * NP;
+            // the next M lines of every group, s of its n done before; groups of a warp that have
+            // fewer (MASK) work on their first rows and store nothing
+            auto step = [&](auto many, auto mask, int s) {
+                constexpr int M = decltype(many)::value;
+                constexpr bool MASK = decltype(mask)::value;
+                float r[M][E];
+#pragma unroll
+                for (int m = 0; m < M; ++m) {
+                    const bool on = !MASK || s + m < n;
+                    const int o = on ? m * ST * NP : 0;
+                    float up[E], bb[E];
+                    if (s + m + 1 < n)
+                        brs::row_ld<E>(up, own + o + NP, lane);
+                    else
+#pragma unroll
+                        for (int q = 0; q < E; ++q)
+                            up[q] = hi[q];
+                    brs::row_ld<E>(bb, brow + o, lane);
+#pragma unroll
+                    for (int q = 0; q < E; ++q)
+                        r[m][q] = PAR ? fma(az, up[q], fma(az, um[q], bb[q]))
+                                      : fma(az, um[q] + up[q], bb[q]);
+                    // the next line's lower neighbour: its old own row (Jacobi), or the row
+                    // above this line (the other parity)
+                    if constexpr (GS) {
+#pragma unroll
+                        for (int q = 0; q < E; ++q)
+                            um[q] = up[q];
+                    } else
+                        brs::row_ld<E>(um, own + o, lane);
+                }
+                brs::line_solve_many<E, G, M>(r, tb, lane);
+#pragma unroll
+                for (int m = 0; m < M; ++m) {
+                    const bool on = !MASK || s + m < n;
+                    float uc[E];
+                    brs::row_ld<E>(uc, own + (on ? m * ST * NP : 0), lane);
+#pragma unroll
+                    for (int q = 0; q < E; ++q)
+                        r[m][q] = fma(tb.wp[q], r[m][q], om1 * uc[q]);
+                    if (on)
+                        brs::row_st<E>(own + m * ST * NP, r[m], lane);
+                }
+                if (!MASK || s + M < n) {
+                    own += M * ST * NP;
+                    brow += M * ST * NP;
+                }
+            };
+            using One = std::integral_constant<int, 1>;
+            using Two = std::integral_constant<int, 2>;
+            int s = 0;
+            if constexpr (G == 32) {
+#pragma unroll 1
+                for (; s + 1 < n; s += 2)
+                    step(Two(), std::false_type(), s);
+                if (s < n)
+                    step(One(), std::false_type(), s);
+            } else {
+                // the groups of a warp step together, as often as the longest run of the CTA
+                const int most = (cnt + NG - 1) / NG;
+#pragma unroll 1
+                for (; s + 1 < most && __any_sync(0xffffffffu, s < n); s += 2)
+                    step(Two(), std::true_type(), s);
+                if (s < most && __any_sync(0xffffffffu, s < n))
+                    step(One(), std::true_type(), s);
             }
+            sync();
+        };
+        for (int it = 0; it < a.nsweeps; ++it) {
+            phase(std::integral_constant<int, 0>());
+            if constexpr (GS)
+                phase(std::integral_constant<int, 1>());
         }
         if (vec) {
             const int n4 = NP / 4;
