@@ -830,12 +830,10 @@ __global__ void split_tf32_kernel(const float* __restrict__ x, float* __restrict
     }
 }
 
-// [k][p][y] -> [k][y][p] through 32 x 32 shared-memory tiles.  SPLIT = 3 / 1: TF32 hi (+ lo)
-// outputs for a tensor-core operand; 0: a plain copy.
-template <typename T, int SPLIT>
+// [k][p][y] -> [k][y][p] through 32 x 32 shared-memory tiles.
+template <typename T>
 __global__ void __launch_bounds__(256) modes_to_rows_kernel(const T* __restrict__ src,
-                                                            T* __restrict__ hi,
-                                                            T* __restrict__ lo, int nm, int ny,
+                                                            T* __restrict__ dst, int nm, int ny,
                                                             int nz)
 {
     __shared__ T tile[32][33];
@@ -854,18 +852,60 @@ __global__ void __launch_bounds__(256) modes_to_rows_kernel(const T* __restrict_
         __syncthreads();
         for (int yy = ty; yy < 32; yy += 8) {
             const int y = y0 + yy, p = p0 + tx;
-            if (p < nm && y < ny) {
-                const T v = tile[tx][yy];
-                const long long o = (long long)k * plane + (long long)y * nm + p;
-                if constexpr (SPLIT == 0) {
-                    hi[o] = v;
-                } else {
-                    const float hb = __uint_as_float(brs_tc::tf32_rn((float)v));
-                    hi[o] = hb;
-                    if (SPLIT == 3)
-                        lo[o] = __uint_as_float(brs_tc::tf32_rn((float)v - hb));
-                }
+            if (p < nm && y < ny)
+                dst[(long long)k * plane + (long long)y * nm + p] = tile[tx][yy];
+        }
+        __syncthreads();
+    }
+}
+
+// The same for a tensor-core operand: TF32 hi and, with SPLIT = 3, lo.  nm and ny are multiples of
+// 32 there, so tiles of 64 x 64 move in 16-byte pieces, four loads of a thread in flight.  Bound by
+// HBM (12 bytes per cell).  256^3, SPLIT = 3, same box: element by element in the tiles above 52.6
+// us (64 instructions per element, 49 % of the issue slots), so 27.4.
+template <int SPLIT>
+__global__ void __launch_bounds__(256) modes_to_split_kernel(const float* __restrict__ src,
+                                                             float* __restrict__ hi,
+                                                             float* __restrict__ lo, int nm,
+                                                             int ny, int nz)
+{
+    __shared__ float tile[64][65];
+    pdl_wait_trigger();
+    const int c = 4 * (threadIdx.x % 16), r = threadIdx.x / 16;
+    const int tiles_y = (ny + 63) / 64;
+    const int y0 = (blockIdx.x % tiles_y) * 64, p0 = (blockIdx.x / tiles_y) * 64;
+    const long long plane = (long long)nm * ny;
+    for (int k = blockIdx.y; k < nz; k += gridDim.y) {
+        float4 v[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int p = p0 + r + 16 * i;
+            if (p < nm && y0 + c < ny)
+                v[i] = __ldg(reinterpret_cast<const float4*>(src + k * plane + (long long)p * ny +
+                                                             y0 + c));
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            float* t = &tile[r + 16 * i][c];
+            t[0] = v[i].x, t[1] = v[i].y, t[2] = v[i].z, t[3] = v[i].w;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int y = y0 + r + 16 * i;
+            if (y >= ny || p0 + c >= nm)
+                continue;
+            float h[4], l[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const float x = tile[c + q][r + 16 * i];
+                h[q] = __uint_as_float(brs_tc::tf32_rn(x));
+                l[q] = __uint_as_float(brs_tc::tf32_rn(x - h[q]));
             }
+            const long long o = k * plane + (long long)y * nm + p0 + c;
+            *reinterpret_cast<float4*>(hi + o) = make_float4(h[0], h[1], h[2], h[3]);
+            if (SPLIT == 3)
+                *reinterpret_cast<float4*>(lo + o) = make_float4(l[0], l[1], l[2], l[3]);
         }
         __syncthreads();
     }
@@ -933,17 +973,15 @@ int modes_inverse(brs_ctx* c, const void* src, void* dst, cudaStream_t s)
         GemmArgs g{};
         g.M = ny; g.N = nx; g.K = nx; g.strideA = plane; g.strideB = 0; g.strideC = plane;
         if (c->p.dtype == BRS_F64) {
-            e = launch_pdl(modes_to_rows_kernel<double, 0>, tgrid, dim3(256), 0, s,
-                           static_cast<const double*>(src), (double*)P->t2, (double*)nullptr, nx,
-                           ny, nz);
+            e = launch_pdl(modes_to_rows_kernel<double>, tgrid, dim3(256), 0, s,
+                           static_cast<const double*>(src), (double*)P->t2, nx, ny, nz);
             if (e == cudaSuccess)
                 e = launch_gemm<double, EPI_STORE>((const double*)P->t2,
                                                    static_cast<const double*>(P->sx),
                                                    static_cast<double*>(dst), g, nz, s);
         } else {
-            e = launch_pdl(modes_to_rows_kernel<float, 0>, tgrid, dim3(256), 0, s,
-                           static_cast<const float*>(src), (float*)P->t2, (float*)nullptr, nx,
-                           ny, nz);
+            e = launch_pdl(modes_to_rows_kernel<float>, tgrid, dim3(256), 0, s,
+                           static_cast<const float*>(src), (float*)P->t2, nx, ny, nz);
             if (e == cudaSuccess)
                 e = launch_gemm<float, EPI_STORE>((const float*)P->t2,
                                                   static_cast<const float*>(P->sx),
@@ -952,12 +990,10 @@ int modes_inverse(brs_ctx* c, const void* src, void* dst, cudaStream_t s)
         return brs_cuda_status(e);
     }
     const int split = P->math == BRS_PLANE_3XTF32 ? 3 : 1;
-    e = split == 3 ? launch_pdl(modes_to_rows_kernel<float, 3>, tgrid, dim3(256), 0, s,
-                                static_cast<const float*>(src), (float*)P->t2, (float*)P->t2_lo,
-                                nx, ny, nz)
-                   : launch_pdl(modes_to_rows_kernel<float, 1>, tgrid, dim3(256), 0, s,
-                                static_cast<const float*>(src), (float*)P->t2, (float*)P->t2_lo,
-                                nx, ny, nz);
+    const dim3 sgrid((unsigned)(((ny + 63) / 64) * ((nx + 63) / 64)), tgrid.y);
+    e = launch_pdl(split == 3 ? modes_to_split_kernel<3> : modes_to_split_kernel<1>, sgrid,
+                   dim3(256), 0, s, static_cast<const float*>(src), (float*)P->t2,
+                   (float*)P->t2_lo, nx, ny, nz);
     if (e != cudaSuccess)
         return brs_cuda_status(e);
     brs_tc::TcArgs g{};
