@@ -34,15 +34,19 @@ struct TwistModeArgs {
 };
 
 // ZC = false: no z coupling and no own value, out = M_p^{-1} b' (the block solve alone).
-template <bool OMEGA1, int DF, int DB, bool ZC>
-__global__ void __launch_bounds__(1024, 1) mode_twist_kernel(
+// SHARE: one CTA per SM takes an equal share of the tasks (launch_twist); else one task per warp.
+template <bool OMEGA1, int DF, int DB, bool ZC, bool SHARE>
+__global__ void __launch_bounds__(SHARE ? 1024 : 256, SHARE ? 1 : 4) mode_twist_kernel(
     const double* uin, double* out, double* zs, const double* __restrict__ bs,
     const double* __restrict__ fm, const double* __restrict__ fb,
     const double* __restrict__ gm, const double* __restrict__ gb, const TwistModeArgs a)
 {
     pdl_wait_trigger();
-    for (long long task = blockIdx.x + (long long)gridDim.x * (threadIdx.x >> 5); task < a.ntasks;
-         task += (long long)gridDim.x * (blockDim.x >> 5)) {
+    long long task = SHARE ? blockIdx.x + (long long)gridDim.x * (threadIdx.x >> 5)
+                           : (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    if (task >= a.ntasks)
+        return;  // warp-uniform
+    do {
     const int lane = threadIdx.x & 31;
     const bool right = lane >= 16;
     const int n = a.ny, m = a.m, nx = a.nx;
@@ -65,12 +69,13 @@ __global__ void __launch_bounds__(1024, 1) mode_twist_kernel(
         const long long o = base + (long long)y * nx;
         const bool q = on && ok;
         v.b = q ? __ldg(bs + o) : 0.0;
-        v.f = q ? __ldg(fm + (long long)ss * nx + p) : 0.0;
         if (ZC) {
             v.zn = (on && fzn) ? __ldg(uin + o - plane) : 0.0;
             v.zp = (on && fzp) ? __ldg(uin + o + plane) : 0.0;
-            v.g = q ? __ldg(fb + (long long)ss * nx + p) : 0.0;
         }
+        v.f = q ? __ldg(fm + (long long)ss * nx + p) : 0.0;
+        if (ZC)
+            v.g = q ? __ldg(fb + (long long)ss * nx + p) : 0.0;
     };
     // elimination towards the twist cell, DF cells of loads in flight
     double z = 0.0;
@@ -98,14 +103,15 @@ __global__ void __launch_bounds__(1024, 1) mode_twist_kernel(
     if (!right) {
         const long long o = base + (long long)m * nx;
         const double bm = ok ? __ldg(bs + o) : 0.0;
-        const double gmv = ok ? __ldg(gm + p) : 0.0;
-        double r = bm;
-        if (ZC) {
+        if constexpr (ZC) {
             const double zn = fzn ? __ldg(uin + o - plane) : 0.0;
             const double zp = fzp ? __ldg(uin + o + plane) : 0.0;
-            r = fma(ok ? __ldg(gb + p) : 0.0, zn + zp, bm);
+            const double gmv = ok ? __ldg(gm + p) : 0.0, gbv = ok ? __ldg(gb + p) : 0.0;
+            y = fma(gmv, z + zr, fma(gbv, zn + zp, bm));
+        } else {
+            const double gmv = ok ? __ldg(gm + p) : 0.0;
+            y = fma(gmv, z + zr, bm);
         }
-        y = fma(gmv, z + zr, r);
         if (ok)
             out[o] = OMEGA1 ? y : fma(a.om1, uin[o], y);
     }
@@ -141,7 +147,8 @@ __global__ void __launch_bounds__(1024, 1) mode_twist_kernel(
             loadb(h, ss + DB, ss + DB < cnt);
         }
     }
-    }  // task
+        task += (long long)gridDim.x * (blockDim.x >> 5);
+    } while (SHARE && task < a.ntasks);
 }
 
 // ---------------------------------------------------------------------------------------
@@ -298,8 +305,11 @@ using TwistModeKernel = void (*)(const double*, double*, double*, const double*,
 // Grids of at least 20 warp tasks per SM: one CTA per SM with an equal share of them, in rounds
 // of at most 32 warps (256^3 has 27 tasks per SM, which 8-warp CTAs, four to an SM, spread as 24
 // or 32: 184 -> 158 us per Jacobi sweep).  Smaller ones keep 8-warp CTAs, which leave SMs free for
-// the next launch's prologue (128^3 calls of 50: 1.84 ms against 2.00 with one CTA per SM).
-int launch_twist(const TwistModeArgs& a, TwistModeKernel k, const double* uin, double* out,
+// the next launch's prologue (128^3 calls of 50: 1.84 ms against 2.00 with one CTA per SM), and
+// one task per warp without the loop over tasks, neighbouring tasks in a CTA (32^3 10.2 us per
+// Jacobi sweep against 11.6 with the loop and spread tasks, 64^3 18.7 against 21.0).
+int launch_twist(const TwistModeArgs& a, TwistModeKernel share_k, TwistModeKernel task_k,
+                 const double* uin, double* out,
                  double* zs, const double* bs, const double* fm, const double* fb, const double* gm,
                  const double* gb, cudaStream_t s)
 {
@@ -315,7 +325,8 @@ int launch_twist(const TwistModeArgs& a, TwistModeKernel k, const double* uin, d
     const bool share = per_sm >= 20;
     const int warps = share ? (int)((per_sm + rounds - 1) / rounds) : 8;
     const unsigned grid = (unsigned)(share ? sms : (a.ntasks + 7) / 8);
-    e = launch_pdl(k, dim3(grid), dim3(32 * warps), 0, s, uin, out, zs, bs, fm, fb, gm, gb, a);
+    e = launch_pdl(share ? share_k : task_k, dim3(grid), dim3(32 * warps), 0, s, uin, out, zs, bs, fm,
+                   fb, gm, gb, a);
     return brs_cuda_status(e);
 }
 
@@ -384,9 +395,12 @@ int mode_twist_launch(const double* uin, double* out, double* zs, const double* 
     const long long planes = colour < 0 ? nz : (nz - colour + 1) / 2;
     a.ntasks = planes * a.npb;
     a.om1 = 1.0 - omega;
-    return launch_twist(a, a.om1 == 0.0 ? mode_twist_kernel<true, 2, 4, true>
-                                        : mode_twist_kernel<false, 2, 4, true>,
-                        uin, out, zs, bs, fm, fb, gm, gb, s);
+    return a.om1 == 0.0 ? launch_twist(a, mode_twist_kernel<true, 2, 4, true, true>,
+                                       mode_twist_kernel<true, 2, 4, true, false>, uin, out, zs, bs,
+                                       fm, fb, gm, gb, s)
+                        : launch_twist(a, mode_twist_kernel<false, 2, 4, true, true>,
+                                       mode_twist_kernel<false, 2, 4, true, false>, uin, out, zs, bs,
+                                       fm, fb, gm, gb, s);
 }
 
 int mode_solve_launch(const double* r, double* out, const double* fm, const double* gm, int nx,
@@ -400,6 +414,7 @@ int mode_solve_launch(const double* r, double* out, const double* fm, const doub
     a.npb = (nx + 15) / 16;
     a.colour = -1;
     a.ntasks = (long long)planes * a.npb;
-    return launch_twist(a, mode_twist_kernel<true, 2, 4, false>, nullptr, out, out, r, fm, nullptr,
-                        gm, nullptr, s);
+    return launch_twist(a, mode_twist_kernel<true, 2, 4, false, true>,
+                        mode_twist_kernel<true, 2, 4, false, false>, nullptr, out, out, r, fm,
+                        nullptr, gm, nullptr, s);
 }
