@@ -519,8 +519,19 @@ def _plane_form(ny):
     return 1 if os.environ.get("BRSMOOTH_PLANE_FORM", "1") == "1" and ny <= 512 else 2
 
 
+def _box_sine_form(box, dt, meth, math):
+    """Whether the library runs these boxes in one pass in the box's sine basis: sides of at
+    most 16, on CUDA cores, or chosen by "auto" where the tensor product's rounding is near."""
+    if os.environ.get("BRSMOOTH_BOX_SINE", "1") == "0" or "BRSMOOTH_BOX_FOLD" in os.environ:
+        return False
+    n = box[0] * box[1] * box[2]
+    cuda_cores = dt == "f64" or math == "simt" or (math == "auto" and (n % 4 or n < 32))
+    near = math == "auto" and n * (2 if meth == "gs" else 1) <= 64
+    return max(box) <= 16 and bool(cuda_cores or near)
+
+
 def _box_fma_per_cell(box, dt, math):
-    """Multiply-adds per cell of the box product as the library runs it: n for the full
+    """Multiply-adds per cell of the dense box product as the library runs it: n for the full
     product; sum over the 8 parity classes of n_c^2 / n on CUDA cores where that saves half
     the work and a class has 16+ cells (BRSMOOTH_BOX_FOLD=0: the full product)."""
     n = box[0] * box[1] * box[2]
@@ -574,12 +585,15 @@ def _variant_grid(brs, stream, barrier, peak, blk, meth, dt, a, steps, sweeps, m
            "sweeps_per_call": sweeps}
     fma = _fma_rate(brs, stream) / 1e9 if dt == "f64" else None
     if blk == "box":
+        out["box"] = list(box)
+        out["plane_math"] = math
+    if blk == "box" and _box_sine_form(box, dt, meth, math):
+        out["box_form"] = "sine basis of the box, one pass per sweep (per colour for GS)"
+    elif blk == "box":
         # the dense block product: n multiply-adds per cell, n = bx by bz (Alg. 2 step 2); on
         # CUDA cores by parity classes where the library uses them: sum_c n_c^2 / n
         nfull = box[0] * box[1] * box[2]
         nb = _box_fma_per_cell(box, dt, math)
-        out["box"] = list(box)
-        out["plane_math"] = math
         out["fma_per_cell"] = nb
         out["parity_classes"] = nb < nfull
         out["tflops"] = rate * 2 * nb / 1e3
@@ -593,29 +607,40 @@ def _variant_grid(brs, stream, barrier, peak, blk, meth, dt, a, steps, sweeps, m
             out["alu_frac_of_fp64_fma_rate"] = rate * nb / fma
     if blk == "plane" and math == "auto":
         math = "3xtf32" if dt == "f32" and N % 32 == 0 else "simt"  # the library's choice
+    # x-transforms by digits on the tensor cores (CUDA-core contexts)
+    digits = (blk == "plane" and math == "simt" and "BRSMOOTH_MODE_FOLD" not in os.environ
+              and os.environ.get("BRSMOOTH_MODE_SLICES", "1") != "0")
     if blk == "plane" and modes:
         # x-sine form: per call, the x-DST of b and of u and the inverse x-DST of u (nx
-        # multiply-adds per cell each; FP64 splits each by the basis's even/odd symmetry into
-        # two half-size products, (ceil(nx/2)^2 + floor(nx/2)^2) / nx per cell), then
-        # mode-line sweeps: 3 words per cell, HBM-bound in FP32
+        # multiply-adds per cell each; by digits on the tensor cores in FP64 and on FP32 CUDA-core
+        # contexts), then mode-line sweeps: 3 words per cell, in FP32 on chip from the first to
+        # the last where a mode fits a cluster
         passes = 3 if math == "3xtf32" else 1
-        fold = dt == "f64" and os.environ.get("BRSMOOTH_MODE_FOLD", "1") != "0"
+        fold = dt == "f64" and not digits and os.environ.get("BRSMOOTH_MODE_FOLD", "1") != "0"
         fma_t = ((N - N // 2) ** 2 + (N // 2) ** 2) / N if fold else float(N)
         out["plane_form"] = "x-sine basis: 3 transforms per call + mode-line sweeps"
         out["plane_math"] = math
+        out["transform_form"] = "digits on the tensor cores" if digits else "products"
         out["transform_fma_per_cell"] = fma_t
         out["tflops"] = 6.0 * fma_t * rate / sweeps / 1e3
         if s_lo < sweeps:
             out["mode_sweep_us"] = sweep_ms * 1e3
             out["mode_sweep_gcell"] = N ** 3 / (sweep_ms / 1e3) / 1e9
-            out["mode_sweep_hbm_frac"] = 3 * es * N ** 3 / (sweep_ms / 1e3) / 1e9 / peak
+            on_chip = (dt == "f32" and N <= 256
+                       and os.environ.get("BRSMOOTH_MODE_RESIDENT", "1") != "0")
+            if on_chip:
+                out["mode_sweep_form"] = "on chip, one mode per cluster"
+                out["hbm_frac_note"] = ("3 words per cell and sweep against the copy rate; the "
+                                        "call moves u and b once for all its sweeps")
+            else:
+                out["mode_sweep_hbm_frac"] = 3 * es * N ** 3 / (sweep_ms / 1e3) / 1e9 / peak
             out["transforms_ms_per_call"] = fixed_ms
             out["transforms_timing"] = (f"calls of {sweeps} and {s_lo} sweeps, the difference "
                                         "per sweep and the remainder per call")
             if math in ("tf32", "3xtf32"):
                 out["transforms_tensor_tflops"] = (3 * 2.0 * N * N ** 3 * passes
                                                    / (fixed_ms / 1e3) / 1e12)
-            if dt == "f64":
+            if dt == "f64" and not digits:
                 out["transforms_frac_of_fp64_fma_rate"] = (3.0 * fma_t * N ** 3
                                                            / (fixed_ms / 1e3) / (fma * 1e9))
     elif blk == "plane":
@@ -635,8 +660,12 @@ def _variant_grid(brs, stream, barrier, peak, blk, meth, dt, a, steps, sweeps, m
             out["tensor_tflops"] = out["tflops"] * passes
             out["tensor_frac_of_tf32_peak"] = out["tensor_tflops"] / tf32_peak
             out["tf32_peak_tflops"] = tf32_peak
-        if dt == "f64":
+        if dt == "f64" and not digits:
             out["alu_frac_of_fp64_fma_rate"] = out["tflops"] / 2 * 1e3 / fma
+    if blk in ("line", "yline", "zline") and dt == "f32" and meth == "jacobi":
+        if os.environ.get("BRSMOOTH_LINE_TWO", "1") != "0":
+            out["hbm_frac_note"] = ("3 words per cell and sweep against the copy rate; a pass "
+                                    "moves them once for two sweeps")
     if blk == "line" and dt == "f64":
         # FP64 pipe roof: 7 operations per cell (6 for Gauss-Seidel with omega = 1, whose
         # update is the solve itself)

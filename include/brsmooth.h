@@ -127,8 +127,11 @@ typedef struct brs_params {
  * xy-plane blocks (BRS_XYPLANE): the plane block is diagonalised along x by the
  * orthonormal DST-I.  FP64 contexts, and FP32 contexts where TMA can stage rows of ny
  * elements (ny times 4 bytes a multiple of 16, ny a whole number of the lane chunks of the
- * line solve), also hold the x-sine form of calls of several sweeps: two more grids (b and
- * u transformed; FP32 [k][p][y], FP64 [k][y][p]) and, for chaotic GS, a third.  Such a call
+ * line solve) or, on CUDA cores, where nx >= 48, also hold the x-sine form of calls of several
+ * sweeps: at most two more grids (b and u transformed; FP32 [k][p][y], FP64 [k][y][p]) and, for
+ * chaotic GS whose sweeps stream (FP32, ny > 256), a third.  CUDA-core contexts of nx >= 48
+ * (FP32: 96) transform by digits on the tensor cores, exact to the type's rounding, and hold the
+ * digits of one block of rows (at most 128 rows per SM, 14 (8) bytes per cell).  Such a call
  * transforms b
  * and u once, runs its sweeps as y-line solves per x-mode with the z coupling, and
  * transforms u back; the iterates are the plane sweeps' own in exact arithmetic (the

@@ -375,10 +375,10 @@ __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_gr
 // u(k+1) and b(k) from its slot and the y neighbours from the slot before, which it then refills.
 // Every patch row is a multiple of 16 bytes (checked on the host).
 // Bound by the latency of a step's chain until enough warps are resident, then by DRAM: 600 patches
-// of 16 to 64 cells a side (38 M cells), us per sweep: with the y neighbours by shuffle and select,
+// of 16 to 64 cells a side (36 M cells), us per sweep: with the y neighbours by shuffle and select,
 // and every row's address formed anew per step, 87 in 118 registers (16 warps per SM, 54 % of the
-// issue slots, DRAM 57 %); so, 82 with 16 warps and 76 with the 20 that 96 registers allow, 0.9 of
-// the copy rate.  24 warps in 80 registers: 78.
+// issue slots, DRAM 57 %); so, 82 with 16 warps and 76 with the 20 that 96 registers allow, 0.84
+// of the copy rate.  24 warps in 80 registers: 78.
 template <int G, bool GS, int D, bool LV>
 __device__ __forceinline__ void batched_item_async(const PatchDesc& d, int jb, int kc, int KC,
                                                    const float* uin, float* uout,
