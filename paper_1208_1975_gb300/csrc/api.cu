@@ -299,7 +299,8 @@ int brsmooth_create(const brs_params* p, brs_ctx** out)
         const char* ev = std::getenv("BRSMOOTH_LINE_SEQ");
         if (rc == BRS_OK && p->dtype == BRS_F64 && !(ev && ev[0] == '0')) {
             rc = line_tile_setup(c);
-            if (rc == BRS_OK && line_seq_takes(c))
+            c->lseq_min = line_seq_min_sweeps(c);
+            if (rc == BRS_OK && c->lseq_min > 0)
                 rc = line_seq_setup(c);
         }
     } else if (p->block == BRS_XYPLANE)
@@ -354,7 +355,7 @@ int brsmooth_sweep(brs_ctx* c, void* u, const void* b, int nsweeps, void* stream
         return batched_sweep(c, u, b, nsweeps, s);
     if (c->perm)
         return perm_sweep(c, u, b, nsweeps, s);
-    if (c->lseq && nsweeps >= kLineSeqMinSweeps)
+    if (c->lseq && nsweeps >= c->lseq_min)
         return line_seq_sweep(c, u, b, nsweeps, s);
     if (c->ltile)
         return line_tile_sweep(c, u, b, nsweeps, s);

@@ -82,7 +82,9 @@ struct brs_ctx {
     float* dc_c = nullptr;
     // adjoint-sweep state (owned by adjoint.cu)
     void* adjoint = nullptr;
-    // FP64 x-line sweeps on the line-major copy (owned by line_seq.cu); null otherwise
+    // FP64 x-line sweeps on the line-major copy (owned by line_seq.cu), for calls of at least
+    // lseq_min sweeps; null otherwise
+    int lseq_min = 0;
     void* lseq = nullptr;
     // FP64 x-line sweeps on the caller's layout (owned by line_tile.cu); null otherwise
     void* ltile = nullptr;
@@ -105,12 +107,8 @@ int line_sweep_launch(brs_ctx* c, const void* uin, void* uout, const void* b, cu
 
 // FP64 x-line path (line_seq.cu): one thread per half line, elimination from both ends,
 // on a line-major colour-split copy of u and b made by each call.
-// Taken for grids of at least 20 16-line tasks per SM in calls of at least 4 sweeps, where the
-// three copies per call are paid back (us per sweep in calls of 1 / 3 / 8 / 30, line-major
-// against line_tile.cu, same box: 256^3 Jacobi 400 / 279 / 240 / 223 against 325 / 293 / 255 /
-// 250; 192^3, 15 tasks per SM, 185 / 130 / 112 / 105 against 151 / 135 / 107 / 105).
-constexpr int kLineSeqMinSweeps = 4;
-bool line_seq_takes(const brs_ctx* c);
+// Sweeps a call needs to take it (0: never; line_tile.cu then takes every call).
+int line_seq_min_sweeps(const brs_ctx* c);
 int line_seq_setup(brs_ctx* c);
 void line_seq_teardown(brs_ctx* c);
 int line_seq_sweep(brs_ctx* c, void* u, const void* b, int nsweeps, cudaStream_t s);

@@ -393,12 +393,39 @@ int pick_shape(brs_ctx* c, long long tasks, bool persist, Shape* sh)
 
 }  // namespace
 
-bool line_seq_takes(const brs_ctx* c)
+// The three copies of a call (c) against a faster sweep than line_tile.cu's: the call is worth them
+// from c / (difference per sweep) sweeps on.  That depends on how full the tile form's chunks of 32
+// cells are, on long lines (it holds fewer), and on the lines per SM, of which the line-major sweep
+// needs enough for its 16-line warps; Gauss-Seidel, with half of them per launch, more.  Measured
+// (us per call, line-major / tile): Jacobi, 320 lines per SM, calls of 3, 4 and 10: 36 cells 121 / 163,
+// 149 / 202, 323 / 497; 48 cells 145 / 163, 184 / 202, 401 / 497; 64 cells 182 / 175, 228 / 216,
+// 513 / 530; 160 cells 431 / 417, 544 / 523, 1215 / 1297; 288 cells 754 / 785, 949 / 992, 2133 /
+// 2477.  100 lines per SM: 64 cells 94 / 73, 120 / 81, 265 / 200.  Gauss-Seidel, 220 lines per SM, calls
+// of 10: 36 cells 325 / 348, 64 cells 499 / 368, 512 cells 4256 / 3952; 800: 64 cells 1118 / 1229.
+int line_seq_min_sweeps(const brs_ctx* c)
 {
-    int sms = 0;
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
     const int force = env_int("BRSMOOTH_LINE_SEQ", 1);  // 2: every grid (measurements, tests)
-    return force == 2 || (long long)c->p.ny * c->p.nz >= 20ll * kLinesPerWarp * sms;
+    if (force == 2)
+        return 4;
+    int sms = 1;
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
+    const long long lines = (long long)c->p.ny * c->p.nz / sms;
+    const int nx = c->p.nx, pad = (nx + 31) / 32 * 32;
+    const bool half = 100 * pad >= 135 * nx, thin = 10 * pad >= 12 * nx, long_ = nx >= 256;
+    if (c->p.method == BRS_JACOBI) {
+        if (half)
+            return lines >= 160 ? 2 : lines >= 130 ? 3 : lines >= 90 ? 4 : 0;
+        if (lines < 160)
+            return 0;
+        return thin || long_ ? 3 : 5;
+    }
+    if (lines < 200)
+        return 0;
+    if (half)
+        return lines < 300 ? 8 : 2;
+    if (thin)
+        return lines < 300 ? 0 : 3;
+    return lines >= (long_ ? 400 : 600) ? 5 : 0;
 }
 
 int line_seq_setup(brs_ctx* c)

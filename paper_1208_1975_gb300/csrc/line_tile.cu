@@ -13,7 +13,7 @@
 // elimination values through L2; and a grid of a few lines per SM spreads its loads and updates
 // over all warps, where two threads per line alone would wait on memory latency.  An FP64 warp
 // instruction occupies its SM quarter for 64 clocks, so the chain warp's place rotates with the
-// CTA.  Calls of few sweeps, and grids of less than about 27 16-line tasks per SM,
+// CTA.  Calls of few sweeps, and grids of few lines per SM (line_seq_min_sweeps),
 // run fastest on it (us per sweep, same box, line-major -> tile): 32^3 Jacobi 12.3 -> 4.4 in calls of
 // 30, 64^3 22.6 -> 9.0, 96^3 32.6 -> 17.5, 128^3 44.7 -> 35.7; Gauss-Seidel 96x88x72 60.1 -> 21.7;
 // 256^3 one-sweep calls 400 -> 325, but 223 -> 250 in calls of 30.  What bounds it at 256^3 is the
@@ -351,7 +351,7 @@ int line_tile_setup(brs_ctx* c)
     if (e == cudaSuccess)
         e = cudaMemcpy(S->tab, tab.data(), tab.size() * sizeof(double), cudaMemcpyHostToDevice);
     // calls of 4 or more sweeps scale b into bs, unless the line-major form takes them
-    if (e == cudaSuccess && !line_seq_takes(c))
+    if (e == cudaSuccess && line_seq_min_sweeps(c) == 0)
         e = cudaMalloc(&S->bs, (size_t)c->cells * sizeof(double));
     a.tab = S->tab;
     const size_t smem = tile_smem(a, kLines);
