@@ -641,7 +641,7 @@ int dst_slices_create(int n, long long rows, int device, int* status, DstSlices<
     // value more exact than a double holds
     const long double pi = 3.14159265358979323846264338327950288L;
     const int per = 2 * (n + 1);
-    std::vector<__nv_bfloat16> dq((size_t)kDig * per);
+    std::vector<__nv_bfloat16> dq((size_t)kDig * per);  // [q][digit]
     std::vector<int> aq((size_t)kDig * per);
     for (int q = 0; q < per; ++q) {
         const long double v = std::sqrt(2.0L / (n + 1)) * std::sin(pi * q / (n + 1));
@@ -649,8 +649,8 @@ int dst_slices_create(int n, long long rows, int device, int* status, DstSlices<
         for (int s = kDig - 1; s >= 0; --s) {
             const int d = s ? (int)(signed char)(m & 255) : (int)m;
             m = (m - d) / 256;
-            dq[(size_t)s * per + q] = __float2bfloat16((float)d);
-            aq[(size_t)s * per + q] = d < 0 ? -d : d;
+            dq[(size_t)q * kDig + s] = __float2bfloat16((float)d);
+            aq[(size_t)q * kDig + s] = d < 0 ? -d : d;
         }
     }
     std::vector<__nv_bfloat16> bd((size_t)kDig * np * Kp, __float2bfloat16(0.0f));
@@ -658,21 +658,22 @@ int dst_slices_create(int n, long long rows, int device, int* status, DstSlices<
     // rows (|d| <= 128).  FP64's lighter ones, from 2^-48 of the largest product down, may round by
     // a few units without reaching FP64's own rounding of the sum.
     for (int p = 0; p < n; ++p) {
-        long long acc = 0;
-        for (int t = 0; t < kDig; ++t) {
-            const __nv_bfloat16* dt = &dq[(size_t)t * per];
-            const int* at = &aq[(size_t)t * per];
-            __nv_bfloat16* row = &bd[((size_t)t * np + p) * Kp];
-            long long sum = 0;  // sum over x of |digit t|
-            for (int x = 0, q = p + 1; x < n; ++x) {
-                row[x] = dt[q];
-                sum += at[q];
-                q += p + 1;
-                if (q >= per)
-                    q -= per;
+        int sum[kDig] = {};  // sums over x of |digit t|
+        for (int x = 0, q = p + 1; x < n; ++x) {
+            const __nv_bfloat16* dt = &dq[(size_t)q * kDig];
+            const int* at = &aq[(size_t)q * kDig];
+            for (int t = 0; t < kDig; ++t) {
+                bd[((size_t)t * np + p) * Kp + x] = dt[t];
+                sum[t] += at[t];
             }
-            acc += 128 * sum;  // weight t + 2 holds the pairs with digits 0 .. t of S
-            if (t < 4 && acc > (1ll << 24))
+            q += p + 1;
+            if (q >= per)
+                q -= per;
+        }
+        long long acc = 0;
+        for (int t = 0; t < 4; ++t) {
+            acc += 128ll * sum[t];  // weight t + 2 holds the pairs with digits 0 .. t of S
+            if (acc > (1ll << 24))
                 return BRS_OK;
         }
     }
