@@ -111,7 +111,8 @@ __device__ __forceinline__ void st_vec(T* p, const T (&v)[W])
 
 // x-rows r0 .. r0 + RPT - 1 (r = ly + by lz) of the block with packed coordinates pk into R row q.
 // The loads of all rows come before the sums of any: row by row, boxes 4 cells wide (two rows per
-// thread) waited for each row in turn (256^3 of 4x8x8, the whole sweep 166 us; 119 so).
+// thread) waited for each row in turn (256^3 of 4x8x8, the whole sweep 166 us; 119 so).  One row per
+// thread loads the x neighbours last: 256^3 of 8x8x8 133.0 us against 134.9 with them first.
 template <typename T, int SPLIT, int BX, int RPT>
 __device__ __forceinline__ void box_gather_rows(const T* __restrict__ u, const T* __restrict__ b,
                                                 T* __restrict__ rhi, float* __restrict__ rlo,
@@ -134,9 +135,9 @@ __device__ __forceinline__ void box_gather_rows(const T* __restrict__ u, const T
         zm |= (unsigned)(lz == 0) << i;
         zp |= (unsigned)(lz == bz - 1) << i;
         ld_vec<T, BX>(v[i], b + cell[i]);
-        if (i0 > 0)
+        if (RPT > 1 && i0 > 0)
             xm[i] = u[cell[i] - 1];
-        if (i0 + BX < nx)
+        if (RPT > 1 && i0 + BX < nx)
             xp[i] = u[cell[i] + BX];
     }
     auto face = [&](unsigned f, bool in, T a, long long off) {
@@ -161,9 +162,9 @@ __device__ __forceinline__ void box_gather_rows(const T* __restrict__ u, const T
 #pragma unroll
     for (int i = 0; i < RPT; ++i) {
         if (i0 > 0)
-            v[i][0] = fma(ax, xm[i], v[i][0]);
+            v[i][0] = fma(ax, RPT > 1 ? xm[i] : u[cell[i] - 1], v[i][0]);
         if (i0 + BX < nx)
-            v[i][BX - 1] = fma(ax, xp[i], v[i][BX - 1]);
+            v[i][BX - 1] = fma(ax, RPT > 1 ? xp[i] : u[cell[i] + BX], v[i][BX - 1]);
         const long long o = q * n + (long long)BX * (r0 + i);
         if constexpr (SPLIT == 0) {
             st_vec<T, BX>(rhi + o, v[i]);
