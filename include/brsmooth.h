@@ -306,8 +306,9 @@ int brsmooth_defect_correction(brs_ctx* outer_f64, brs_ctx* inner_f32, double* u
  * blocks, dM/dax = Tx, dM/day = dM/daz = 2I.  Calls for sweeps K-1 .. 0 in that order
  * give dL/du_0 in `lam`, dL/db in grad_b and dL/da in grad_a.  The context owns one more
  * grid buffer and reduction scratch, allocated on first use; the Jacobi scratch buffer
- * is reused.  Errors: BRS_ERR_ARG (null), BRS_ERR_UNSUPPORTED (not a single-grid x-line
- * block-Jacobi context), BRS_ERR_NOMEM, BRS_ERR_CUDA.
+ * is reused.  Errors: BRS_ERR_ARG (null; an array not aligned to its elements; u_k or b not
+ * aligned to 16 bytes on a grid whose rows TMA can stage), BRS_ERR_UNSUPPORTED (not a
+ * single-grid x-line block-Jacobi context), BRS_ERR_NOMEM, BRS_ERR_CUDA.
  */
 int brsmooth_adjoint_sweep(brs_ctx* c, void* lam, const void* u_k, const void* b,
                            void* grad_b, double* grad_a, void* stream);

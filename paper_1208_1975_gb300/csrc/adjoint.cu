@@ -556,6 +556,13 @@ extern "C" int brsmooth_adjoint_sweep(brs_ctx* c, void* lam, const void* u_k, co
         return BRS_ERR_ARG;
     if (c->batch || c->p.block != BRS_XLINE || c->p.method != BRS_JACOBI)
         return BRS_ERR_UNSUPPORTED;
+    // whole elements; u_k and b from a 16-byte boundary where TMA can stage the rows (FP32 loads them
+    // so; FP64 reads single elements, but takes the same arrays)
+    auto misaligned = [](const void* q, size_t to) { return reinterpret_cast<uintptr_t>(q) % to != 0; };
+    const size_t in = c->lcfg.tma ? 16 : c->esize;
+    if (misaligned(lam, c->esize) || misaligned(grad_b, c->esize) || misaligned(u_k, in) ||
+        misaligned(b, in) || misaligned(grad_a, sizeof(double)))
+        return BRS_ERR_ARG;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     if (!c->adjoint) {
         AdjState* A = new AdjState();
