@@ -1,0 +1,74 @@
+"""FP64 box sweeps in the box's sine basis against extended precision: no further from it than the
+dense inverse (products of 64 to 512 terms) is, at sides whose transforms scale a sine to 1 (2, 4, 8)
+and others, and at coefficients that weigh the axes differently."""
+import numpy as np
+import pytest
+
+from test_gpu_box import brs, gpu_sweeps  # noqa: F401
+
+pytestmark = pytest.mark.gpu
+
+BOXES = [(8, 8, 8), (2, 2, 2), (4, 4, 4), (4, 2, 2), (8, 8, 4), (6, 5, 4), (3, 3, 3), (16, 4, 2)]
+COEFFS = [(1.0, 1.0, 1.0), (1.0, 0.1, 0.01), (0.5, 1.0, 2.0)]
+LD = np.longdouble
+PI = LD(4) * np.arctan(LD(1))
+
+
+def along(M, x, axis):
+    return np.moveaxis(np.moveaxis(x, axis, -1) @ M.T, -1, axis)
+
+
+def exact(u, b, a, box, omega, method, sweeps):
+    """The sweeps in extended precision, by the sine basis of the boxes."""
+    u, b, a = u.astype(LD), b.astype(LD), [LD(v) for v in a]
+    S = [np.sqrt(LD(2) / (n + 1)) * np.sin(np.outer(np.arange(1, n + 1), np.arange(1, n + 1)) * PI / (n + 1))
+         for n in box]
+    eig = [4 * np.sin(np.arange(1, n + 1) * PI / (2 * (n + 1))) ** 2 for n in box]
+    lam = a[0] * eig[0][None, None, :] + a[1] * eig[1][None, :, None] + a[2] * eig[2][:, None, None]
+    nz, ny, nx = u.shape
+    cut = (nz // box[2], box[2], ny // box[1], box[1], nx // box[0], box[0])
+    at = np.indices((cut[0], cut[2], cut[4])).sum(axis=0) % 2
+
+    def correction(v):
+        r = b - 2 * (a[0] + a[1] + a[2]) * v
+        for axis, c in ((2, a[0]), (1, a[1]), (0, a[2])):
+            w = np.moveaxis(v, axis, 0)
+            s = np.zeros_like(w)
+            s[1:] += w[:-1]
+            s[:-1] += w[1:]
+            r = r + c * np.moveaxis(s, 0, axis)
+        t = r.reshape(cut).transpose(0, 2, 4, 1, 3, 5)
+        for d in range(3):
+            t = along(S[d], t, 5 - d)
+        t = t / lam
+        for d in range(3):
+            t = along(S[d], t, 5 - d)
+        return t  # [box z, y, x][cell z, y, x]
+
+    for _ in range(sweeps):
+        for colour in ((None,) if method == "jacobi" else (0, 1)):
+            t = LD(omega) * correction(u)
+            if colour is not None:
+                t = np.where((at == colour)[..., None, None, None], t, LD(0))
+            u = u + t.transpose(0, 3, 1, 4, 2, 5).reshape(u.shape)
+    return u
+
+
+@pytest.mark.parametrize("method,omega,sweeps", [("jacobi", 0.8, 5), ("gs", 1.0, 3)])
+@pytest.mark.parametrize("a", COEFFS, ids=str)
+@pytest.mark.parametrize("box", BOXES, ids=lambda s: "x".join(map(str, s)))
+def test_no_further_than_the_dense_inverse(brs, box, a, method, omega, sweeps, monkeypatch):  # noqa: F811
+    n = [-(-20 // v) * v for v in box]
+    rng = np.random.default_rng(11)
+    u = rng.uniform(-1, 1, (n[2], n[1], n[0]))
+    b = rng.uniform(-1, 1, u.shape) / (n[0] + 1) ** 2
+    ref = exact(u, b, a, box, omega, method, sweeps)
+
+    def distance():
+        got = gpu_sweeps(brs, u, b, a, box, dt="f64", method=method, omega=omega, math="simt",
+                         nsweeps=sweeps)[-1]
+        return float(np.sqrt(((got.astype(LD) - ref) ** 2).sum() / (ref ** 2).sum()))
+
+    sine = distance()
+    monkeypatch.setenv("BRSMOOTH_BOX_SINE", "0")
+    assert sine <= distance()
