@@ -286,29 +286,29 @@ __global__ void __launch_bounds__(kThreads, 2) adjoint_update_march(
 
 // FP64 form: lanes along x, a warp marches over kc planes of 32 cells of a row with mu of planes
 // k-1, k, k+1 in registers and the next plane's inputs in flight.  Bound by the FP64 pipe, so it
-// counts operations, 15 per cell instead of 22, by two identities of the symmetric operators:
-//   A mu = M mu - (ay Sy + az Sz) mu and M mu = lambda, so
-//     lambda <- (1 - omega) lambda + omega (ay Sy + az Sz) mu   (no x neighbours, no diagonal);
-//   mu . Tx x = (Tx mu) . x and mu . Sd u = (Sd mu) . u, so the sums need the neighbours of mu
-//     only, which the first line has: (2 mu - Sx mu) x, 2 mu x - (Sy mu) u, 2 mu x - (Sz mu) u,
-//     differences formed cell by cell as before.
+// counts operations, 17 per cell instead of 22: mu . Tx x = (Tx mu) . x and mu . Sd u = (Sd mu) . u,
+// so the sums need the neighbours of mu only, which A mu has: (2 mu - Sx mu) x, 2 mu x - (Sy mu) u,
+// 2 mu x - (Sz mu) u, differences formed cell by cell as before.  (A mu = M mu - (ay Sy + az Sz) mu
+// with M mu = lambda would save two more, lambda <- (1 - omega) lambda + omega (ay Sy + az Sz) mu, but
+// it carries the block solve's rounding along: grad_u0 after 8 sweeps 1.2 to 1.6 times as far from
+// extended precision as with A mu itself, 40x30x20 and 33x24x25, for 4 % of a call's time.)
 // The last CTA to finish adds the CTAs' sums into grad_a in a fixed order (a counter in global
-// memory, left at zero for the next call).  128^3, same box: 109 -> 74 us per call.
+// memory, left at zero for the next call).  128^3, same box: 109 -> 82 us per call.
 struct StepIn {
     double mup, muym, muyp, mul, mur, lam, x, u, gb;
 };
 
 __global__ void __launch_bounds__(kThreads, 3) adjoint_update_f64(
     double* __restrict__ lam, const double* __restrict__ mu, const double* __restrict__ x,
-    const double* __restrict__ u, double* __restrict__ gb, int nx, int ny, int nz, int kc, double oy,
-    double oz, double omega, double* partials, unsigned* counter, double* grad_a)
+    const double* __restrict__ u, double* __restrict__ gb, int nx, int ny, int nz, int kc, double ax,
+    double ay, double az, double omega, double* partials, unsigned* counter, double* grad_a)
 {
     pdl_wait_trigger();
     const long long plane = (long long)nx * ny;
     const int ncx = (nx + 31) / 32, nkc = (nz + kc - 1) / kc;
     const long long nitems = (long long)ny * ncx * nkc;
     const int lane = threadIdx.x & 31, wpb = blockDim.x >> 5;
-    const double om1 = 1.0 - omega;
+    const double dg = 2.0 * (ax + ay + az);
     double g0 = 0.0, g1 = 0.0, g2 = 0.0;
     for (long long it = (long long)blockIdx.x * wpb + (threadIdx.x >> 5); it < nitems;
          it += (long long)gridDim.x * wpb) {
@@ -338,7 +338,8 @@ __global__ void __launch_bounds__(kThreads, 3) adjoint_update_f64(
             if (k + 1 < k1)
                 load(nxt, o + plane, k + 1);
             const double sy = c.muym + c.muyp, sz = mum + c.mup, sx = c.mul + c.mur;
-            const double lv = fma(oz, sz, fma(oy, sy, om1 * c.lam));
+            const double off = fma(ax, sx, fma(az, sz, ay * sy));
+            const double lv = fma(omega, fma(-dg, muc, off), c.lam);  // lam - omega A mu
             const double gv = fma(omega, muc, c.gb);
             const double m2 = muc + muc, t = m2 * c.x;
             g0 = fma(m2 - sx, c.x, g0);
@@ -498,7 +499,7 @@ int adjoint_run_f64(brs_ctx* c, double* lam, const double* u, const double* b, d
     }
     return brs_cuda_status(launch_pdl(adjoint_update_f64, dim3(A->nblocks), dim3(kThreads), 0, s,
                                       lam, (const double*)mu, (const double*)x, u, gb, p.nx, p.ny,
-                                      p.nz, kc, c->omega * p.ay, c->omega * p.az, c->omega,
+                                      p.nz, kc, p.ax, p.ay, p.az, c->omega,
                                       A->partials, A->counter, ga));
 }
 
