@@ -16,6 +16,7 @@
 #include <cstdlib>
 #include <map>
 #include <mutex>
+#include <tuple>
 #include <vector>
 
 #include "batched.cuh"
@@ -888,6 +889,9 @@ int env_int(const char* name, int dflt)
     return (v && *v) ? std::atoi(v) : dflt;
 }
 
+// z-chunk fixed by the environment (0: none); a level stages at most kMaxKC z-steps of x ghosts.
+int fixed_chunk() { return std::min(std::max(env_int("BRSMOOTH_BATCH_KC", 0), 0), kMaxKC); }
+
 // The cp.async rings of every resident warp fit one SM.
 bool async_fits(const BatchState* B, int warps, int ctas_per_sm, bool level)
 {
@@ -905,16 +909,18 @@ void set_shape(brs_ctx* c, int warps, int ctas_per_sm)
 }
 
 // Autotuner: time each candidate (z-chunk, warps per CTA, CTAs per SM) on scratch
-// arrays of the real patch set and keep the fastest.  Results are cached per process
-// keyed by the patch set, dtype and method.
+// arrays of the real patch set and keep the fastest.  Results are cached per process, keyed by
+// all that decides which candidates there are and how fast they run: the device, the patch set,
+// dtype, method, the kernel and its ring, and a chunk length fixed by BRSMOOTH_BATCH_KC.
 struct TuneKey {
     std::vector<int> dims;
-    int dtype, method;
+    int device, dtype, method;
+    int stages;  // cp.async ring slots; 0: direct loads
+    int kc;      // fixed z-chunk; 0: any
     bool operator<(const TuneKey& o) const
     {
-        if (dtype != o.dtype) return dtype < o.dtype;
-        if (method != o.method) return method < o.method;
-        return dims < o.dims;
+        return std::tie(device, dtype, method, stages, kc, dims) <
+               std::tie(o.device, o.dtype, o.method, o.stages, o.kc, o.dims);
     }
 };
 struct TuneVal {
@@ -926,7 +932,8 @@ std::mutex g_tune_mutex;
 int autotune(brs_ctx* c)
 {
     BatchState* B = bs(c);
-    TuneKey key{B->dims, c->p.dtype, c->p.method};
+    const int fixed_kc = fixed_chunk();
+    TuneKey key{B->dims, c->device, c->p.dtype, c->p.method, B->async ? B->stages : 0, fixed_kc};
     {
         std::lock_guard<std::mutex> lk(g_tune_mutex);
         auto it = g_tune_cache.find(key);
@@ -935,10 +942,8 @@ int autotune(brs_ctx* c)
             return build_items(c, it->second.KC);
         }
     }
-    int fixed_kc = env_int("BRSMOOTH_BATCH_KC", 0);
-    fixed_kc = fixed_kc > kMaxKC ? kMaxKC : fixed_kc;
     std::vector<TuneVal> cands;
-    for (int kc : {4, 8, 16, 32})
+    for (int kc : fixed_kc ? std::vector<int>{fixed_kc} : std::vector<int>{4, 8, 16, 32})
         for (int w : {4, 8, 16})
             for (int cps : {2, 4, 5, 8}) {
                 if (w * cps > 64 || (!B->async && cps == 5))
@@ -946,8 +951,6 @@ int autotune(brs_ctx* c)
                 // cp.async kernel: 8 or 20 warps per SM in CTAs of 4 warps, 16 in CTAs of 8
                 if (B->async && (w * 32 > kAsyncThreads || cps == 4 ||
                                  !async_fits(B, w, cps, false)))
-                    continue;
-                if (fixed_kc && kc != fixed_kc)
                     continue;
                 cands.push_back({kc, w, cps});
             }
@@ -968,7 +971,7 @@ int autotune(brs_ctx* c)
         cudaEventCreate(&e0);
         cudaEventCreate(&e1);
     }
-    TuneVal best{8, 8, 4};
+    TuneVal best = cands[0];
     float best_ms = 1e30f;
     for (const TuneVal& v : cands) {
         if (rc != BRS_OK)
@@ -1092,9 +1095,8 @@ int batched_setup(brs_ctx* c, int npatch, const int* dims)
                 return brs_cuda_status(e);
         }
     }
-    int kc = env_int("BRSMOOTH_BATCH_KC", 0);
-    kc = kc > kMaxKC ? kMaxKC : kc;  // a level stages at most kMaxKC z-steps of x ghosts
     if (env_int("BRSMOOTH_BATCH_NOTUNE", 0)) {
+        const int kc = fixed_chunk();
         set_shape(c, 8, B->async ? 2 : 4);
         return build_items(c, kc ? kc : 8);
     }
