@@ -116,31 +116,33 @@ typedef struct brs_params {
  * FP64 x-line blocks: each line is eliminated from both ends by two threads with pivots
  * factored once (Sec. 2 / Sec. 4.3: invert once, reuse), on the caller's arrays (the context
  * holds one grid-sized buffer for b scaled by the pivots).  Grids of many lines (from 90 to
- * 600 per SM on, by their length and the method) hold three buffers of nx*nz*2*ceil(ny/2) doubles
- * instead: calls of several sweeps (2 to 8 at least, likewise) run on line-major copies there (cell index i outermost, the lines of each row k split by colour
- * (j+k) mod 2), u and b copied in and u back per call (three grid passes).  Both forms do the
- * same operations in the same order: the iterates are the same bit for bit.
+ * 600 per SM on, by their length and the method) hold three buffers of nx*nz*2*ceil(ny/2)
+ * doubles instead: calls of several sweeps (2 to 8 at least, likewise) run on line-major copies
+ * there (cell index i outermost, the lines of each row k split by colour (j+k) mod 2), u and b
+ * copied in and u back per call (three grid passes).  Both forms do the same operations in the
+ * same order: the iterates are the same bit for bit.
  * Chaotic GS on these contexts visits the lines in two colours, j+k even then odd, each
  * colour reading the other colour's newest values: the red-black line order, one
  * admissible order of the chaotic scheme, deterministic.  BRSMOOTH_LINE_SEQ=0 in the
  * environment at creation selects the lane-scan kernel of the FP32 path instead.
  * xy-plane blocks (BRS_XYPLANE): the plane block is diagonalised along x by the
- * orthonormal DST-I.  FP64 contexts, and FP32 contexts where TMA can stage rows of ny
- * elements (ny times 4 bytes a multiple of 16, ny a whole number of the lane chunks of the
- * line solve) or, on CUDA cores, where nx >= 48, also hold the x-sine form of calls of several
- * sweeps: at most two more grids (b and u transformed; FP32 [k][p][y], FP64 [k][y][p]) and, for
- * chaotic GS whose sweeps stream (FP32, ny > 256), a third.  CUDA-core contexts of nx >= 48
- * (FP32: 96) transform by digits on the tensor cores, exact to the type's rounding, and hold the
- * digits of one block of rows (at most 128 rows per SM, 14 (8) bytes per cell).  Such a call
- * transforms b
- * and u once, runs its sweeps as y-line solves per x-mode with the z coupling, and
- * transforms u back; the iterates are the plane sweeps' own in exact arithmetic (the
- * transform commutes with the sweep), rounded differently, so a call of n sweeps is not
- * bitwise equal to n one-sweep calls.  It is taken for calls of at least 3 sweeps on the
- * tensor-core path and at least 2 otherwise (BRSMOOTH_PLANE_MODES_MIN); BRSMOOTH_PLANE_MODES=0
- * in the environment at creation leaves it out.  FP64 solves each y-line by elimination from
- * both ends (BRSMOOTH_MODE_TWIST=0: the lane-scan solve, TMA rows only).  Chaotic GS on plane contexts visits the
- * planes in two colours, even k then odd k, each colour reading the other's newest values.
+ * orthonormal DST-I.  CUDA-core contexts of nx = 48 (FP32: 96) to 511, 503 excepted, and
+ * ny <= 512 transform by digits on the tensor cores, exact to the type's rounding of each row's
+ * 2-norm, and hold the digits of one block of rows (at most 128 rows per SM, 14 (8) bytes per
+ * cell); other rows are transformed by products in the type.
+ * FP64 contexts, and FP32 contexts where TMA can stage rows of ny elements (ny times 4 bytes a
+ * multiple of 16, ny a whole number of the lane chunks of the line solve) or, on CUDA cores,
+ * where nx >= 48, also hold the x-sine form of calls of several sweeps: at most two more grids
+ * (b and u transformed; FP32 [k][p][y], FP64 [k][y][p]) and, for chaotic GS whose sweeps stream
+ * (FP32, ny > 256), a third.  Such a call transforms b and u once, runs its sweeps as y-line
+ * solves per x-mode with the z coupling, and transforms u back; the iterates are the plane
+ * sweeps' own in exact arithmetic (the transform commutes with the sweep), rounded differently,
+ * so a call of n sweeps is not bitwise equal to n one-sweep calls.  It is taken for calls of at
+ * least 3 sweeps on the tensor-core path and at least 2 otherwise (BRSMOOTH_PLANE_MODES_MIN);
+ * BRSMOOTH_PLANE_MODES=0 in the environment at creation leaves it out.  FP64 solves each y-line
+ * by elimination from both ends (BRSMOOTH_MODE_TWIST=0: the lane-scan solve, TMA rows only).
+ * Chaotic GS on plane contexts visits the planes in two colours, even k then odd k, each colour
+ * reading the other's newest values.
  */
 int brsmooth_create(const brs_params* p, brs_ctx** out);
 

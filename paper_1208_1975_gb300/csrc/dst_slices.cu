@@ -9,9 +9,18 @@
 //   x = 2^e sum_s d_s 2^(-8 s),  |d_s| <= 128,  s = 1..7   (56 bits; e from the row's largest)
 // and the digit products are summed on the tensor cores in bf16 with FP32 accumulators, which hold
 // integers below 2^24 exactly.  Products of equal weight, s + t = const, share an accumulator; the
-// 28 pairs with s + t <= 8 reach below FP64's rounding of the row's largest product (the ones left
-// out are under 2^-72 of it each).  One output is 7 exact integers, joined in 64-bit integer
-// arithmetic and rounded: no FP64 instruction at all per output.
+// 28 pairs with s + t <= 8 are summed.  A pair left out is at most 2^-58 of 2^(e + eb), the scale of
+// the row's digits and S's, which is 4 to 16 times the row's largest product: the six of weight 9 come
+// to at most 6 n 2^-58 of it, and as digits fall to about (6 n)^(1/2) 2^-60 (2^-55 at n = 256), where a
+// product on the FP64 pipe rounds n/2 partial sums by up to 2^-53 each.  One output is 7 exact
+// integers, joined in 64-bit integer arithmetic and rounded: no FP64 instruction at all per output.
+// Rows of wide range keep the 2-norm error of the others (one spike, decaying cells, random exponents
+// over 3 to 30 decades, n = 130: FP64 1.7 .. 2.9e-16 against 5.1 .. 7.1e-16 by products, FP32 6 .. 8e-8
+// against 2.4 .. 3.9e-7).
+//
+// Rows of n = 48 (FP32 96) to 511 values, 503 excepted.  From 512 on S's largest value falls below the
+// next power of two, eb drops with it, and the sums of the first four weights could pass 2^24 (1.18
+// times at 512); those of 503 could by its digits (1.07 times).
 //
 // Measured at 256^3, same box: 0.41 ms per transform (0.07 slicing, 0.34 products, whose digit
 // tiles, 84 KB per 56 instructions, come from L2 at about 7 TB/s) against 3.6; calls of 50 FP64
