@@ -470,13 +470,16 @@ void fill_args(SineArgs<T>& a, const brs_params& p, double omega)
     a.om1 = (T)(1.0 - omega);
 }
 
+// Eigenvalue 2 - 2 cos((q+1) pi / (n+1)) = 4 sin^2 of half the angle.
+long double eig(int n, int q)
+{
+    const long double sine = basis(2 * n + 1, q + 1);
+    return 4.0L * (n + 1) * sine * sine;
+}
+
 template <typename T>
 int upload_ilam(void** dst, const brs_params& p, double omega)
 {
-    auto eig = [](int m, int q) {  // 2 - 2 cos((q+1) pi / (m+1)) = 4 sin^2 of half the angle
-        const long double sine = basis(2 * m + 1, q + 1);
-        return 4.0L * (m + 1) * sine * sine;
-    };
     const long double k = kappa(p.bx) * kappa(p.by) * kappa(p.bz);
     std::vector<T> v;
     for (int r = 0; r < p.bz; ++r)

@@ -731,13 +731,12 @@ void dst_slices_destroy(DstSlices<T>* d)
     delete d;
 }
 
-template <typename T>
-int dst_slices_run(const DstSlices<T>* d, const T* src, T* dst, const T* scale, int period,
-                   long long rows, cudaStream_t s)
+int dst_slices_run(const DstSlices<double>* d, const double* src, double* dst, const double* scale,
+                   int period, long long rows, cudaStream_t s)
 {
-    RowSource<T> rs{};
+    RowSource<double> rs{};
     rs.src = src;
-    SliceArgs<T> g{};
+    SliceArgs<double> g{};
     g.dst = dst;
     g.scale = scale;
     g.period = period;
@@ -809,8 +808,6 @@ int dst_slices_from_modes(const DstSlices<float>* d, const float* src, float* ds
 #define BRS_DST_SLICES(T)                                                                      \
     template int dst_slices_create<T>(int, long long, int, int*, DstSlices<T>**);               \
     template void dst_slices_destroy<T>(DstSlices<T>*);                                         \
-    template int dst_slices_run<T>(const DstSlices<T>*, const T*, T*, const T*, int, long long, \
-                                   cudaStream_t);                                               \
     template int dst_slices_rhs<T>(const DstSlices<T>*, const T*, const T*, double, T*, const T*, \
                                    int, int, int, int, int, bool, cudaStream_t);                \
     template int dst_slices_update<T>(const DstSlices<T>*, const T*, const T*, double, double,  \

@@ -18,11 +18,10 @@ int dst_slices_create(int n, long long rows, int device, int* status, DstSlices<
 template <typename T>
 void dst_slices_destroy(DstSlices<T>* d);
 
-// dst[row][p] = sum_x S[p][x] src[row][x], times scale[(row % period) * n + p] if scale is set.
+// FP64: dst[row][p] = sum_x S[p][x] src[row][x], times scale[(row % period) * n + p] if scale is set.
 // src and dst: [rows][n], not overlapping.
-template <typename T>
-int dst_slices_run(const DstSlices<T>* d, const T* src, T* dst, const T* scale, int period,
-                   long long rows, cudaStream_t s);
+int dst_slices_run(const DstSlices<double>* d, const double* src, double* dst, const double* scale,
+                   int period, long long rows, cudaStream_t s);
 
 // The same transform of the plane right-hand sides R_k = b_k + az (u_{k-1} + u_{k+1}) (zero outside
 // the grid) of planes k0, k0 + kstep, ... of [nz][ny][n] grids: dst[plane][y][p], planes packed,

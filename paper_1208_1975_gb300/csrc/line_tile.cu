@@ -251,8 +251,10 @@ size_t tile_smem(const TileArgs& a, int nl) { return (size_t)nl * a.pitch * size
 template <int MODE, int LPU>
 const void* tile_kernel(bool om1)
 {
-    return om1 ? (const void*)xline_tile_kernel<true, MODE, LPU>
-               : (const void*)xline_tile_kernel<false, MODE, LPU>;
+    if constexpr (MODE != SOLVE_ONLY)  // a block solve has no own value to keep
+        if (!om1)
+            return (const void*)xline_tile_kernel<false, MODE, LPU>;
+    return (const void*)xline_tile_kernel<true, MODE, LPU>;
 }
 
 const void* tile_kernel(int mode, int lpu, bool om1)

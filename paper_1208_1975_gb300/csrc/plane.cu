@@ -1356,7 +1356,7 @@ int twist_sweep(brs_ctx* c, void* u, const void* b, int nsweeps, cudaStream_t s,
                             static_cast<const double*>(P->tscale), ny, rows, s);
         if (rc == BRS_OK)
             rc = u_zero ? brs_cuda_status(cudaMemsetAsync(mu, 0, (size_t)c->cells * sizeof(double), s))
-                        : dst_slices_run<double>(P->slices, static_cast<const double*>(u), mu, nullptr, 1,
+                        : dst_slices_run(P->slices, static_cast<const double*>(u), mu, nullptr, 1,
                                          rows, s);
     } else if (P->fold) {
         rc = dst_fold_forward(static_cast<const double*>(b), mb,
@@ -1394,7 +1394,7 @@ int twist_sweep(brs_ctx* c, void* u, const void* b, int nsweeps, cudaStream_t s,
         }
     }
     if (rc == BRS_OK && P->slices)
-        return dst_slices_run<double>(P->slices, cur, static_cast<double*>(u), nullptr, 1, rows, s);
+        return dst_slices_run(P->slices, cur, static_cast<double*>(u), nullptr, 1, rows, s);
     if (rc == BRS_OK)
         rc = P->fold ? dst_fold_inverse(cur, static_cast<double*>(u), w1, w2,
                                         static_cast<const double*>(P->tSeT),
