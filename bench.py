@@ -6,7 +6,9 @@ library call of 50 sweeps.  With N ranks (torchrun) every rank sweeps its own re
 data-path collective: the grids are independent), so `value` is N x cells x sweeps /
 (max-over-ranks time).
 
-Also reported on the same JSON line:
+Printed on one JSON line, short enough for a log that keeps its last few thousand characters;
+everything measured, with the notes and each variant in full, goes to a file (--details,
+bench_details.json beside this script unless given).  On the line, besides the value:
   roofline     -- the binding roof of the FP64 sweep kernel: FP64 pipe operations (7 per
                   cell: gather 4, elimination 1 each way, update 1) per launch / average
                   launch time, against the FP64 FMA rate measured in the same run;
@@ -15,8 +17,10 @@ Also reported on the same JSON line:
                   copies of u and b and the D2H copy of u inside the timed region;
   cpu_baseline -- the FP64 CPU oracle on the host cores on a bounded slab of the grid;
   clocks       -- nvidia-smi samples taken during the timed region;
-  variants     -- other method / dtype / coefficient / block combinations, each with its
-                  error against the FP64 oracle and, where timed, the oracle's own rate.
+  variants     -- how many other method / dtype / coefficient / block combinations ran, which
+                  failed, how many errors were taken against the FP64 oracle and which are
+                  beyond their tolerance (in the file: each with its rate, its error and,
+                  where timed, the oracle's own rate).
 
 `--impl reference` times the FP64 CPU oracle instead (rank 0 only), on the same metric.
 """
@@ -1442,6 +1446,42 @@ def _variants(brs, stream, barrier, peak):
     return out
 
 
+def _oracle_errors(v):
+    """(value, tolerance) of every error against the oracle in a variant's record."""
+    if isinstance(v, list):
+        return [e for x in v for e in _oracle_errors(x)]
+    if not isinstance(v, dict):
+        return []
+    out = [e for x in v.values() for e in _oracle_errors(x)]
+    if "tolerance" in v:
+        out += [(x, v["tolerance"]) for k, x in v.items()
+                if k != "tolerance" and isinstance(x, float)]
+    return out
+
+
+def headline(full, details):
+    """The line to print: the full record without its notes, the variants counted."""
+    keep = {"roofline": ("bound", "achieved", "peak", "unit", "frac", "traffic", "kernel",
+                         "launch_ms"),
+            "roofline_hbm": ("achieved", "peak", "unit", "frac"),
+            "cpu_baseline": ("value", "unit", "cores", "kind"),
+            "e2e": ("value", "unit", "h2d_bytes_per_step", "d2h_bytes_per_step", "steps")}
+    line = {}
+    for k, v in full.items():
+        if k in keep and v is not None:
+            v = {q: v[q] for q in keep[k]}
+        if k not in ("gpu_launches_note", "variants"):
+            line[k] = v
+    names = {id(v): str(v.get("name") or v.get("workload"))[:40] for v in full["variants"]}
+    errors = [(names[id(v)], e, t) for v in full["variants"] for e, t in _oracle_errors(v)]
+    line["variants"] = {"run": len(full["variants"]),
+                        "failed": [names[id(v)] for v in full["variants"] if "error" in v],
+                        "oracle_errors": len(errors),
+                        "beyond_tolerance": sorted({n for n, e, t in errors if not e <= t})}
+    line["details"] = details
+    return line
+
+
 def main():
     ap = argparse.ArgumentParser()
     ap.add_argument("--gpus", type=int, default=1)
@@ -1452,6 +1492,8 @@ def main():
     ap.add_argument("--no-cpu", action="store_true")
     ap.add_argument("--only", default=None,
                     help="run one named workload variant and print its JSON (for profiling)")
+    ap.add_argument("--details", default=str(ROOT / "bench_details.json"),
+                    help="file for the full record (the printed line is its summary)")
     args = ap.parse_args()
     args.warmup = max(args.warmup, 3)
     if args.impl == "reference":
@@ -1582,7 +1624,12 @@ def main():
                                  "1 copy back",
             "roofline": roofline, "roofline_hbm": roofline_hbm, "cpu_baseline": cpu,
             "e2e": e2e, "clocks": clocks, "variants": variants}
-    print(json.dumps(line), flush=True)
+    details = args.details
+    try:
+        Path(details).write_text(json.dumps(line, indent=1) + "\n")
+    except OSError as exc:
+        details = f"not written: {exc}"[:200]
+    print(json.dumps(headline(line, details)), flush=True)
     if ws > 1:
         import torch.distributed as dist
 
