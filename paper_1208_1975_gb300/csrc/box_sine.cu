@@ -442,9 +442,18 @@ void fill_args(SineArgs<T>& a, const brs_params& p, double omega)
 {
     const int n[3] = {p.bx, p.by, p.bz};
     for (int d = 0; d < 3; ++d) {
-        for (int q = 0; q < n[d]; ++q)
-            for (int i = 0; i < (q % 2 ? n[d] / 2 : (n[d] + 1) / 2); ++i)
-                (q % 2 ? a.o : a.e)[d][(q / 2) * kHalf + i] = (T)basis(n[d], (q + 1) * (i + 1));
+        if (n[d] != 2 && n[d] != 4 && n[d] != 8) {
+            const int m = n[d] + 1;
+            std::vector<T> sine(2 * m);  // basis of every product of indexes, mod its period
+            for (int q = 1; 2 * q <= m; ++q) {
+                sine[q] = sine[m - q] = (T)basis(n[d], q);
+                sine[m + q] = sine[2 * m - q] = -sine[q];
+            }
+            for (int q = 0; q < n[d]; ++q)
+                for (int i = 0; i < (q % 2 ? n[d] / 2 : (n[d] + 1) / 2); ++i)
+                    (q % 2 ? a.o : a.e)[d][(q / 2) * kHalf + i] =
+                        sine[(q + 1) * (i + 1) % (2 * m)];
+        }
         if (n[d] == 4)
             a.e[d][0] = (T)(basis(4, 2) / kappa(4));
         if (n[d] == 8) {
@@ -470,23 +479,48 @@ void fill_args(SineArgs<T>& a, const brs_params& p, double omega)
     a.om1 = (T)(1.0 - omega);
 }
 
-// Eigenvalue 2 - 2 cos((q+1) pi / (n+1)) = 4 sin^2 of half the angle.
-long double eig(int n, int q)
+// A value of extended precision as the sum of two doubles.
+struct Two {
+    double hi, lo;
+    explicit Two(long double v) : hi((double)v), lo((double)(v - hi)) {}
+};
+
+// s / (a + b) to a rounding of the last place, in double arithmetic (extended precision runs in
+// software on Arm).
+double quotient(const Two& s, const Two& a, const Two& b)
 {
-    const long double sine = basis(2 * n + 1, q + 1);
-    return 4.0L * (n + 1) * sine * sine;
+    const double h = a.hi + b.hi, t = h - a.hi;
+    const double l = ((a.hi - (h - t)) + (b.hi - t)) + (a.lo + b.lo);  // a + b = h + l
+    const double q = s.hi / h;
+    return q + (std::fma(-q, h, s.hi) + (s.lo - q * l)) / h;
+}
+
+// Eigenvalues 2 - 2 cos((q+1) pi / (n+1)) = 4 sin^2 of half the angle, times a.
+std::vector<long double> eigenvalues(int n, double a)
+{
+    std::vector<long double> v(n);
+    for (int q = 0; q < n; ++q) {
+        const long double sine = basis(2 * n + 1, q + 1);
+        v[q] = a * 4.0L * (n + 1) * sine * sine;
+    }
+    return v;
 }
 
 template <typename T>
 int upload_ilam(void** dst, const brs_params& p, double omega)
 {
+    const std::vector<long double> x = eigenvalues(p.bx, p.ax), y = eigenvalues(p.by, p.ay),
+                                   z = eigenvalues(p.bz, p.az);
+    const std::vector<Two> x2(x.begin(), x.end());
     const long double k = kappa(p.bx) * kappa(p.by) * kappa(p.bz);
+    const Two scale(omega * k * k);
     std::vector<T> v;
     for (int r = 0; r < p.bz; ++r)
-        for (int q = 0; q < p.by; ++q)
+        for (int q = 0; q < p.by; ++q) {
+            const Two yz(y[q] + z[r]);
             for (int i = 0; i < p.bx; ++i)
-                v.push_back((T)(omega * k * k / (p.ax * eig(p.bx, i) + p.ay * eig(p.by, q) +
-                                         p.az * eig(p.bz, r))));
+                v.push_back((T)quotient(scale, x2[i], yz));
+        }
     cudaError_t e = cudaMalloc(dst, v.size() * sizeof(T));
     if (e == cudaSuccess)
         e = cudaMemcpy(*dst, v.data(), v.size() * sizeof(T), cudaMemcpyHostToDevice);
