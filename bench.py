@@ -1331,7 +1331,8 @@ VARIANTS.update({
     "plane_jacobi_f32_tf32_aniso": ("plane", "jacobi", "f32", ANISO, 4, 50, "tf32"),
     "plane_jacobi_f32_simt_aniso": ("plane", "jacobi", "f32", ANISO, 2, 50, "simt"),
     # the per-sweep form of the plane solve (two tensor-core products per sweep), which
-    # calls of one or two sweeps run (BRSMOOTH_PLANE_MODES=0 below)
+    # calls of one or two sweeps run (BRSMOOTH_PLANE_MODES=0 below; FP64 by FP64 products then,
+    # where its one-sweep calls transform by digits)
     "plane_jacobi_f32_aniso_per_sweep": ("plane", "jacobi", "f32", ANISO, 4, 10, "auto"),
     "plane_gs_f32_aniso_per_sweep": ("plane", "gs", "f32", ANISO, 4, 10, "auto"),
     "plane_jacobi_f32_tf32_aniso_per_sweep": ("plane", "jacobi", "f32", ANISO, 4, 10, "tf32"),

@@ -15,7 +15,7 @@
 // cluster barriers per sweep order all of it.  The operations on a cell are those of
 // mode_tma_kernel, in its order, so the results are the same bit for bit.  Rows are padded to
 // G E cells with zeros (zero table entries keep them zero), so any ny up to 512 does.
-// Bound by the latency of a phase, two lines per warp and a cluster barrier: 40 % of the issue
+// Bound by the latency of a phase, two lines per warp and a cluster barrier: 34 % of the issue
 // slots, most stalls on shared memory and the scans' shuffles.  Two lines are solved side by side,
 // because one line's chain leaves most of its warp's issue slots empty (24 -> 20.7 us per sweep).
 // Where a line takes the whole warp, a warp's share of the planes is warp-uniform and it steps
