@@ -25,6 +25,7 @@
 //
 // Taken for boxes whose sides are at most 16: a side of N costs N/2 + 1 operations per cell and
 // transform, and a line of N cells has to fit a thread's registers.
+#include <algorithm>
 #include <cmath>
 #include <new>
 #include <type_traits>
@@ -52,8 +53,22 @@ struct SineArgs {
     T ax, ay, az, om1;
 };
 
+// omega / lambda of a mode over the squared norms of its basis rows: FP32 as a sum of two, whose
+// rounding would otherwise stay in that mode sweep after sweep (2^3 to 16x4x2 boxes: mean error 1.15
+// times the dense FP32 inverse's without the second part, 1.07 with it).
+template <typename T>
+struct ModeScale {
+    using type = T;
+};
+template <>
+struct ModeScale<float> {
+    using type = float2;
+};
+__device__ __forceinline__ double times(double v, double s) { return v * s; }
+__device__ __forceinline__ float times(float v, float2 s) { return fma(v, s.x, v * s.y); }
+
 struct SineState {
-    void* ilam = nullptr;  // omega kappa^2 / lambda_pqr, p fastest (context dtype)
+    void* ilam = nullptr;  // ModeScale per mode, p fastest
     SineArgs<double> a64;
     SineArgs<float> a32;
     size_t smem = 0;
@@ -102,7 +117,8 @@ __device__ __forceinline__ void st_line(T* p, const T (&v)[N])
 }
 
 // v <- S v / kappa (N = 2, 4, 8: kappa scales one sine of the basis to 1, which turns its
-// products into sums; kappa = 1 otherwise).  S is symmetric, so this is the transform back, too.
+// products into sums; otherwise 1 / kappa is FP32's best_scale, or 1).  S is symmetric, so this is the
+// transform back, too.
 // Operations per cell: 1, 2, 3.75 for N = 2, 4, 8, and N/2 + 1 by the two half-size products.
 template <typename T, int N>
 __device__ __forceinline__ void dst(T (&v)[N], const T* e, const T* o)
@@ -198,7 +214,7 @@ __global__ void __launch_bounds__(kThreads) box_sine_kernel(const T* u, T* uout,
                                                             const T* __restrict__ b,
                                                             const long long* __restrict__ rows,
                                                             long long M,
-                                                            const T* __restrict__ ilam,
+                                                            const typename ModeScale<T>::type* __restrict__ ilam,
                                                             const __grid_constant__ SineArgs<T> a)
 {
     extern __shared__ __align__(16) unsigned char box_smem[];
@@ -302,7 +318,7 @@ __global__ void __launch_bounds__(kThreads) box_sine_kernel(const T* u, T* uout,
             dst<T, N>(v, a.e[2], a.o[2]);
 #pragma unroll
             for (int m = 0; m < N; ++m)
-                v[m] *= __ldg(ilam + m * bxy + c);
+                v[m] = times(v[m], __ldg(ilam + m * bxy + c));
             dst<T, N>(v, a.e[2], a.o[2]);
 #pragma unroll
             for (int m = 0; m < N; ++m)
@@ -431,36 +447,79 @@ long double basis(int n, int q)
     return std::sqrt(2.0L / (n + 1)) * std::sin(q * pi / (n + 1));
 }
 
-// 1 / kappa of dst(): the sine that is scaled to 1 (times the basis' norm) for N = 2, 4, 8.
-long double kappa(int n)
+// An axis of the basis as the kernel has it: scaled and rounded.  The squared norms of its rows, as
+// they are, go into the modes' scale: norm of row 0, and norm / (norm of row p) - 1.
+struct Axis {
+    long double norm = 1.0L;
+    std::vector<double> off;
+};
+
+// Scale in [1, 2) at which the sines of an axis lose least to rounding to FP32: every product of the
+// basis takes it, and the modes' scale takes it out.
+double best_scale(int n)
 {
-    return n == 2 || n == 4 ? basis(n, 1) : n == 8 ? basis(n, 3) : 1.0L;
+    std::vector<double> sine;
+    for (int q = 1; 2 * q <= n + 1; ++q)
+        sine.push_back((double)basis(n, q));
+    double best = 1.0, least = 1.0;
+    for (int j = 0; j < 2048; ++j) {
+        const double scale = 1.0 + j / 2048.0;
+        double worst = 0.0;
+        for (size_t q = 0; q < sine.size() && worst < least; ++q) {
+            const double x = scale * sine[q];
+            worst = std::max(worst, std::fabs((double)(float)x - x) / x);
+        }
+        if (worst < least)
+            least = worst, best = scale;
+    }
+    return best;
+}
+
+// e / o of one axis of n cells (see dst for n = 2, 4, 8).
+template <typename T>
+Axis fill_axis(int n, T* e, T* o)
+{
+    Axis ax;
+    ax.off.assign(n, 0.0);
+    auto sq = [](long double v) { return v * v; };
+    if (n == 2) {
+        ax.norm = 2.0L;
+    } else if (n == 4) {
+        e[0] = (T)(basis(4, 2) / basis(4, 1));
+        ax.norm = 2.0L * (1.0L + sq(e[0]));
+    } else if (n == 8) {
+        e[0] = (T)(basis(8, 1) / basis(8, 3));
+        e[1] = (T)(basis(8, 2) / basis(8, 3));
+        ax.norm = 2.0L * (sq(e[0]) + sq(e[1]) + sq((long double)e[0] + e[1]) + 1.0L);
+        ax.off[2] = ax.off[5] = (double)(ax.norm / 6.0L - 1.0L);  // the rows of sin(60) and 0
+    } else if (n > 1) {
+        const int m = n + 1;
+        const double scale = sizeof(T) == 4 ? best_scale(n) : 1.0;
+        std::vector<T> sine(2 * m);  // basis of every product of indexes, mod its period
+        for (int q = 1; 2 * q <= m; ++q) {
+            sine[q] = sine[m - q] = (T)(scale * basis(n, q));
+            sine[m + q] = sine[2 * m - q] = -sine[q];
+        }
+        std::vector<long double> norm(n, 0.0L);
+        for (int q = 0; q < n; ++q)
+            for (int i = 0; i < (q % 2 ? n / 2 : (n + 1) / 2); ++i) {
+                const T v = sine[(q + 1) * (i + 1) % (2 * m)];
+                (q % 2 ? o : e)[(q / 2) * kHalf + i] = v;
+                norm[q] += sq(v) * (2 * i + 1 == n ? 1 : 2);  // once for the middle cell
+            }
+        ax.norm = norm[0];
+        for (int q = 0; q < n; ++q)
+            ax.off[q] = (double)(norm[0] / norm[q] - 1.0L);
+    }
+    return ax;
 }
 
 template <typename T>
-void fill_args(SineArgs<T>& a, const brs_params& p, double omega)
+void fill_args(SineArgs<T>& a, const brs_params& p, double omega, Axis (&axes)[3])
 {
     const int n[3] = {p.bx, p.by, p.bz};
-    for (int d = 0; d < 3; ++d) {
-        if (n[d] != 2 && n[d] != 4 && n[d] != 8) {
-            const int m = n[d] + 1;
-            std::vector<T> sine(2 * m);  // basis of every product of indexes, mod its period
-            for (int q = 1; 2 * q <= m; ++q) {
-                sine[q] = sine[m - q] = (T)basis(n[d], q);
-                sine[m + q] = sine[2 * m - q] = -sine[q];
-            }
-            for (int q = 0; q < n[d]; ++q)
-                for (int i = 0; i < (q % 2 ? n[d] / 2 : (n[d] + 1) / 2); ++i)
-                    (q % 2 ? a.o : a.e)[d][(q / 2) * kHalf + i] =
-                        sine[(q + 1) * (i + 1) % (2 * m)];
-        }
-        if (n[d] == 4)
-            a.e[d][0] = (T)(basis(4, 2) / kappa(4));
-        if (n[d] == 8) {
-            a.e[d][0] = (T)(basis(8, 1) / kappa(8));
-            a.e[d][1] = (T)(basis(8, 2) / kappa(8));
-        }
-    }
+    for (int d = 0; d < 3; ++d)
+        axes[d] = fill_axis(n[d], a.e[d], a.o[d]);
     a.bx = p.bx, a.by = p.by, a.bz = p.bz;
     a.nx = p.nx, a.ny = p.ny, a.nz = p.nz;
     // Threads and boxes per CTA: boxes until the stage with the fewest lines has one per thread
@@ -506,24 +565,33 @@ std::vector<long double> eigenvalues(int n, double a)
     return v;
 }
 
+void put(std::vector<double>& v, double s) { v.push_back(s); }
+void put(std::vector<float2>& v, double s)
+{
+    v.push_back(make_float2((float)s, (float)(s - (float)s)));
+}
+
 template <typename T>
-int upload_ilam(void** dst, const brs_params& p, double omega)
+int upload_ilam(void** dst, const brs_params& p, double omega, const Axis (&axes)[3])
 {
     const std::vector<long double> x = eigenvalues(p.bx, p.ax), y = eigenvalues(p.by, p.ay),
                                    z = eigenvalues(p.bz, p.az);
     const std::vector<Two> x2(x.begin(), x.end());
-    const long double k = kappa(p.bx) * kappa(p.by) * kappa(p.bz);
-    const Two scale(omega * k * k);
-    std::vector<T> v;
+    const Two scale(omega / (axes[0].norm * axes[1].norm * axes[2].norm));
+    std::vector<typename ModeScale<T>::type> v;
     for (int r = 0; r < p.bz; ++r)
         for (int q = 0; q < p.by; ++q) {
             const Two yz(y[q] + z[r]);
-            for (int i = 0; i < p.bx; ++i)
-                v.push_back((T)quotient(scale, x2[i], yz));
+            const double off = axes[1].off[q] + axes[2].off[r];
+            for (int i = 0; i < p.bx; ++i) {
+                const double s = quotient(scale, x2[i], yz);
+                put(v, std::fma(s, axes[0].off[i] + off, s));
+            }
         }
-    cudaError_t e = cudaMalloc(dst, v.size() * sizeof(T));
+    const size_t bytes = v.size() * sizeof(v[0]);
+    cudaError_t e = cudaMalloc(dst, bytes);
     if (e == cudaSuccess)
-        e = cudaMemcpy(*dst, v.data(), v.size() * sizeof(T), cudaMemcpyHostToDevice);
+        e = cudaMemcpy(*dst, v.data(), bytes, cudaMemcpyHostToDevice);
     return brs_cuda_status(e);
 }
 
@@ -534,8 +602,8 @@ int launch(const SineState* S, const SineArgs<T>& a, const void* u, void* uout, 
     const T* up = static_cast<const T*>(u);
     T* op = static_cast<T*>(uout);
     const T* bp = static_cast<const T*>(b);
-    const T* il = static_cast<const T*>(S->ilam);
-    void* args[] = {&up, &op, &bp, (void*)&rows, &M, &il, (void*)&a};
+    const void* il = S->ilam;
+    void* args[] = {&up, &op, &bp, (void*)&rows, &M, (void*)&il, (void*)&a};
     const long long ctas = (M + a.nb - 1) >> a.lognb;
     return brs_cuda_status(launch_pdl_c(S->kernel, dim3((unsigned)ctas), dim3(a.threads), S->smem,
                                         s, args));
@@ -556,15 +624,16 @@ int box_sine_setup(const brs_params& p, double omega, void** out)
     *out = S;
     int rc;
     int nb, Q;
+    Axis axes[3];
     if (p.dtype == BRS_F64) {
-        fill_args(S->a64, p, omega);
-        rc = upload_ilam<double>(&S->ilam, p, omega);
+        fill_args(S->a64, p, omega, axes);
+        rc = upload_ilam<double>(&S->ilam, p, omega, axes);
         S->kernel = sine_kernel_for<double>(p.bx, p.by, p.bz);
         nb = S->a64.nb, Q = S->a64.Q;
         S->smem = (size_t)nb * Q * 8;
     } else {
-        fill_args(S->a32, p, omega);
-        rc = upload_ilam<float>(&S->ilam, p, omega);
+        fill_args(S->a32, p, omega, axes);
+        rc = upload_ilam<float>(&S->ilam, p, omega, axes);
         S->kernel = sine_kernel_for<float>(p.bx, p.by, p.bz);
         nb = S->a32.nb, Q = S->a32.Q;
         S->smem = (size_t)nb * Q * 4;

@@ -1,9 +1,11 @@
-"""FP64 box sweeps in the box's sine basis against extended precision: no further from it than the
-dense inverse (products of 64 to 512 terms) is, at sides whose transforms scale a sine to 1 (2, 4, 8)
-and others, and at coefficients that weigh the axes differently."""
+"""Box sweeps in the box's sine basis against extended precision, beside the dense inverse (products of
+64 to 512 terms): FP64 no further from it, FP32 no more than a rounding further, at sides whose
+transforms scale a sine to 1 (2, 4, 8) and others, and at coefficients that weigh the axes
+differently."""
 import numpy as np
 import pytest
 
+from gpu_common import rounded
 from test_gpu_box import brs, gpu_sweeps  # noqa: F401
 
 pytestmark = pytest.mark.gpu
@@ -54,21 +56,39 @@ def exact(u, b, a, box, omega, method, sweeps):
     return u
 
 
-@pytest.mark.parametrize("method,omega,sweeps", [("jacobi", 0.8, 5), ("gs", 1.0, 3)])
-@pytest.mark.parametrize("a", COEFFS, ids=str)
-@pytest.mark.parametrize("box", BOXES, ids=lambda s: "x".join(map(str, s)))
-def test_no_further_than_the_dense_inverse(brs, box, a, method, omega, sweeps, monkeypatch):  # noqa: F811
+def distances(lib, box, a, dt, method, omega, sweeps, monkeypatch):
+    """2-norm distances from extended precision: in the sine basis, by the dense inverse."""
     n = [-(-20 // v) * v for v in box]
     rng = np.random.default_rng(11)
-    u = rng.uniform(-1, 1, (n[2], n[1], n[0]))
-    b = rng.uniform(-1, 1, u.shape) / (n[0] + 1) ** 2
+    u = rounded(rng.uniform(-1, 1, (n[2], n[1], n[0])), dt)
+    b = rounded(rng.uniform(-1, 1, u.shape) / (n[0] + 1) ** 2, dt)
     ref = exact(u, b, a, box, omega, method, sweeps)
 
     def distance():
-        got = gpu_sweeps(brs, u, b, a, box, dt="f64", method=method, omega=omega, math="simt",
+        got = gpu_sweeps(lib, u, b, a, box, dt=dt, method=method, omega=omega, math="simt",
                          nsweeps=sweeps)[-1]
         return float(np.sqrt(((got.astype(LD) - ref) ** 2).sum() / (ref ** 2).sum()))
 
     sine = distance()
     monkeypatch.setenv("BRSMOOTH_BOX_SINE", "0")
-    assert sine <= distance()
+    return sine, distance()
+
+
+@pytest.mark.parametrize("method,omega,sweeps", [("jacobi", 0.8, 5), ("gs", 1.0, 3)])
+@pytest.mark.parametrize("a", COEFFS, ids=str)
+@pytest.mark.parametrize("box", BOXES, ids=lambda s: "x".join(map(str, s)))
+def test_no_further_than_the_dense_inverse(brs, box, a, method, omega, sweeps, monkeypatch):  # noqa: F811
+    sine, dense = distances(brs, box, a, "f64", method, omega, sweeps, monkeypatch)
+    assert sine <= dense
+
+
+@pytest.mark.parametrize("method,omega,sweeps", [("jacobi", 0.8, 5), ("gs", 1.0, 3)])
+@pytest.mark.parametrize("a", COEFFS + [(1.0, 1.0, 0.01)], ids=str)
+@pytest.mark.parametrize("box", BOXES + [(5, 5, 5), (7, 3, 1), (12, 3, 5)],
+                         ids=lambda s: "x".join(map(str, s)))
+def test_fp32_beside_the_dense_inverse(brs, box, a, method, omega, sweeps, monkeypatch):  # noqa: F811
+    """The kernel's operations emulated on the CPU, over these boxes, coefficients and methods, come to
+    0.6 .. 1.63 times the dense inverse's error, 1.07 on average, at which exact constants would leave
+    them, too (1.10).  A tenth more is allowed for other fields."""
+    sine, dense = distances(brs, box, a, "f32", method, omega, sweeps, monkeypatch)
+    assert sine <= 1.8 * dense
