@@ -109,10 +109,87 @@ __device__ __forceinline__ void st_vec(T* p, const T (&v)[W])
     }
 }
 
-// x-rows r0 .. r0 + RPT - 1 (r = ly + by lz) of the block with packed coordinates pk into R row q.
-// The loads of all rows come before the sums of any: row by row, boxes 4 cells wide (two rows per
-// thread) waited for each row in turn (256^3 of 4x8x8, the whole sweep 166 us; 119 so).  One row per
-// thread loads the x neighbours last: 256^3 of 8x8x8 133.0 us against 134.9 with them first.
+template <typename T, int BX>
+__device__ __forceinline__ void add_row(T (&v)[BX], T a, const T (&t)[BX])
+{
+#pragma unroll
+    for (int m = 0; m < BX; ++m)
+        v[m] = fma(a, t[m], v[m]);
+}
+
+// One row of R, as the product takes it.
+template <typename T, int SPLIT, int BX>
+__device__ __forceinline__ void box_store_row(T* __restrict__ rhi, float* __restrict__ rlo, long long o,
+                                              const T (&v)[BX])
+{
+    if constexpr (SPLIT == 0) {
+        st_vec<T, BX>(rhi + o, v);
+    } else {
+        float h[BX], l[BX];
+#pragma unroll
+        for (int m = 0; m < BX; ++m) {
+            const uint32_t hb = brs_tc::tf32_rn((float)v[m]);
+            h[m] = __uint_as_float(hb);
+            l[m] = __uint_as_float(brs_tc::tf32_rn((float)v[m] - h[m]));
+        }
+        st_vec<float, BX>(rhi + o, h);
+        if (SPLIT == 3)
+            st_vec<float, BX>(rlo + o, l);
+    }
+}
+
+// x-row r (r = ly + by lz) of the block with packed coordinates pk into R row q.  The loads come before
+// the sums: a row has one neighbour row in y and one in z at most (two only in a block one cell thick),
+// and small grids wait for each trip to memory.  Each face loaded and added in turn, in 32 registers
+// instead of 40, us per split-TF32 sweep, same box: 64^3 of 8x8x4 14.4 against 13.9 so, 160x68x16 of
+// 8x4x4 Gauss-Seidel 25.9 against 25.1; 256^3 of 8x8x8 133.6 against 134.4, Gauss-Seidel 177.2
+// against 174.9.
+template <typename T, int SPLIT, int BX>
+__device__ __forceinline__ void box_gather_row(const T* __restrict__ u, const T* __restrict__ b,
+                                               T* __restrict__ rhi, float* __restrict__ rlo,
+                                               long long q, long long pk, int r, int n, int by,
+                                               int bz, int nx, int ny, int nz, long long plane,
+                                               T ax, T ay, T az)
+{
+    const int ly = r % by, lz = r / by;  // uniform per CTA
+    const int i0 = (int)(pk & 0x1FFFFF) * BX;
+    const int j = (int)((pk >> 21) & 0x1FFFFF) * by + ly, k = (int)(pk >> 42) * bz + lz;
+    const long long cell = i0 + (long long)nx * j + plane * k;
+    const bool yl = ly == 0 && j > 0, yh = ly == by - 1 && j + 1 < ny;
+    const bool zl = lz == 0 && k > 0, zh = lz == bz - 1 && k + 1 < nz;
+    const bool xl = i0 > 0, xh = i0 + BX < nx;
+    T v[BX], y[BX], z[BX], xm = T(0), xp = T(0);
+    ld_vec<T, BX>(v, b + cell);
+    if (yl || yh)
+        ld_vec<T, BX>(y, u + cell + (yl ? -nx : nx));
+    if (zl || zh)
+        ld_vec<T, BX>(z, u + cell + (zl ? -plane : plane));
+    if (xl)
+        xm = u[cell - 1];
+    if (xh)
+        xp = u[cell + BX];
+    if (yl || yh)
+        add_row(v, ay, y);
+    if (yl && yh) {
+        ld_vec<T, BX>(y, u + cell + nx);
+        add_row(v, ay, y);
+    }
+    if (zl || zh)
+        add_row(v, az, z);
+    if (zl && zh) {
+        ld_vec<T, BX>(z, u + cell + plane);
+        add_row(v, az, z);
+    }
+    if (xl)
+        v[0] = fma(ax, xm, v[0]);
+    if (xh)
+        v[BX - 1] = fma(ax, xp, v[BX - 1]);
+    box_store_row<T, SPLIT, BX>(rhi, rlo, q * n + (long long)BX * r, v);
+}
+
+// x-rows r0 .. r0 + RPT - 1 of a block into R row q.  The loads of all rows come before the sums of any:
+// row by row, boxes 4 cells wide (two rows per thread) waited for each row in turn (256^3 of 4x8x8,
+// the whole sweep 166 us; 119 so).
 template <typename T, int SPLIT, int BX, int RPT>
 __device__ __forceinline__ void box_gather_rows(const T* __restrict__ u, const T* __restrict__ b,
                                                 T* __restrict__ rhi, float* __restrict__ rlo,
@@ -123,6 +200,7 @@ __device__ __forceinline__ void box_gather_rows(const T* __restrict__ u, const T
     const int i0 = (int)(pk & 0x1FFFFF) * BX;
     const int jb = (int)((pk >> 21) & 0x1FFFFF) * by, kb = (int)(pk >> 42) * bz;
     const long long base = i0 + (long long)nx * jb + plane * kb;
+    const bool xl = i0 > 0, xh = i0 + BX < nx;
     T v[RPT][BX], xm[RPT], xp[RPT];
     long long cell[RPT];
     unsigned ym = 0, yp = 0, zm = 0, zp = 0;  // rows on each face of the block, uniform per CTA
@@ -135,9 +213,9 @@ __device__ __forceinline__ void box_gather_rows(const T* __restrict__ u, const T
         zm |= (unsigned)(lz == 0) << i;
         zp |= (unsigned)(lz == bz - 1) << i;
         ld_vec<T, BX>(v[i], b + cell[i]);
-        if (RPT > 1 && i0 > 0)
+        if (xl)
             xm[i] = u[cell[i] - 1];
-        if (RPT > 1 && i0 + BX < nx)
+        if (xh)
             xp[i] = u[cell[i] + BX];
     }
     auto face = [&](unsigned f, bool in, T a, long long off) {
@@ -151,9 +229,7 @@ __device__ __forceinline__ void box_gather_rows(const T* __restrict__ u, const T
 #pragma unroll
         for (int i = 0; i < RPT; ++i)
             if (f >> i & 1)
-#pragma unroll
-                for (int m = 0; m < BX; ++m)
-                    v[i][m] = fma(a, t[i][m], v[i][m]);
+                add_row(v[i], a, t[i]);
     };
     face(ym, jb > 0, ay, -nx);
     face(yp, jb + by < ny, ay, nx);
@@ -161,25 +237,11 @@ __device__ __forceinline__ void box_gather_rows(const T* __restrict__ u, const T
     face(zp, kb + bz < nz, az, plane);
 #pragma unroll
     for (int i = 0; i < RPT; ++i) {
-        if (i0 > 0)
-            v[i][0] = fma(ax, RPT > 1 ? xm[i] : u[cell[i] - 1], v[i][0]);
-        if (i0 + BX < nx)
-            v[i][BX - 1] = fma(ax, RPT > 1 ? xp[i] : u[cell[i] + BX], v[i][BX - 1]);
-        const long long o = q * n + (long long)BX * (r0 + i);
-        if constexpr (SPLIT == 0) {
-            st_vec<T, BX>(rhi + o, v[i]);
-        } else {
-            float h[BX], l[BX];
-#pragma unroll
-            for (int m = 0; m < BX; ++m) {
-                const uint32_t hb = brs_tc::tf32_rn((float)v[i][m]);
-                h[m] = __uint_as_float(hb);
-                l[m] = __uint_as_float(brs_tc::tf32_rn((float)v[i][m] - h[m]));
-            }
-            st_vec<float, BX>(rhi + o, h);
-            if (SPLIT == 3)
-                st_vec<float, BX>(rlo + o, l);
-        }
+        if (xl)
+            v[i][0] = fma(ax, xm[i], v[i][0]);
+        if (xh)
+            v[i][BX - 1] = fma(ax, xp[i], v[i][BX - 1]);
+        box_store_row<T, SPLIT, BX>(rhi, rlo, q * n + (long long)BX * (r0 + i), v[i]);
     }
 }
 
@@ -207,8 +269,12 @@ __global__ void __launch_bounds__(256) box_gather_kernel(
         return;
     const long long pk = __ldg(rows + q);
     const long long plane = (long long)nx * ny;
-    box_gather_rows<T, SPLIT, BX, RPT>(u, b, rhi, rlo, q, pk, r0, n, by, bz, nx, ny, nz, plane, ax,
-                                       ay, az);
+    if constexpr (RPT == 1)
+        box_gather_row<T, SPLIT, BX>(u, b, rhi, rlo, q, pk, r0, n, by, bz, nx, ny, nz, plane, ax, ay,
+                                     az);
+    else
+        box_gather_rows<T, SPLIT, BX, RPT>(u, b, rhi, rlo, q, pk, r0, n, by, bz, nx, ny, nz, plane,
+                                           ax, ay, az);
 }
 
 // The same for any bx (one cell per loop step, scalar accesses).
