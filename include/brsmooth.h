@@ -115,9 +115,9 @@ typedef struct brs_params {
  * as for x-lines, and nz <= 65535 (y-lines) or ny <= 65535 (z-lines).
  * FP64 x-line blocks: each line is eliminated from both ends by two threads with pivots
  * factored once (Sec. 2 / Sec. 4.3: invert once, reuse), on the caller's arrays (the context
- * holds one grid-sized buffer for b scaled by the pivots).  Grids of many lines (from 90 to
- * 600 per SM on, by their length and the method) hold three buffers of nx*nz*2*ceil(ny/2)
- * doubles instead: calls of several sweeps (2 to 8 at least, likewise) run on line-major copies
+ * holds one grid-sized buffer for b scaled by the pivots).  Grids of many lines (from 88 to
+ * 520 per SM on, by their length and the method) hold three buffers of nx*nz*2*ceil(ny/2)
+ * doubles instead: calls of several sweeps (2 to 20 at least, likewise) run on line-major copies
  * there (cell index i outermost, the lines of each row k split by colour (j+k) mod 2), u and b
  * copied in and u back per call (three grid passes).  Both forms do the same operations in the
  * same order: the iterates are the same bit for bit.

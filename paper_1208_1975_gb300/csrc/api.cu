@@ -302,6 +302,8 @@ int brsmooth_create(const brs_params* p, brs_ctx** out)
             c->lseq_min = line_seq_min_sweeps(c);
             if (rc == BRS_OK && c->lseq_min > 0)
                 rc = line_seq_setup(c);
+            if (rc == BRS_OK && c->lseq)
+                line_tile_borrow(c, line_seq_b(c));
         }
     } else if (p->block == BRS_XYPLANE)
         rc = plane_setup(c);

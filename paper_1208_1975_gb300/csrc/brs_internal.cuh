@@ -110,6 +110,8 @@ int line_sweep_launch(brs_ctx* c, const void* uin, void* uout, const void* b, cu
 // Sweeps a call needs to take it (0: never; line_tile.cu then takes every call).
 int line_seq_min_sweeps(const brs_ctx* c);
 int line_seq_setup(brs_ctx* c);
+// Its buffer for scaled b, at least nx ny nz doubles, free between its calls.
+double* line_seq_b(brs_ctx* c);
 void line_seq_teardown(brs_ctx* c);
 int line_seq_sweep(brs_ctx* c, void* u, const void* b, int nsweeps, cudaStream_t s);
 

@@ -393,15 +393,22 @@ int pick_shape(brs_ctx* c, long long tasks, bool persist, Shape* sh)
 
 }  // namespace
 
-// The three copies of a call (c) against a faster sweep than line_tile.cu's: the call is worth them
-// from c / (difference per sweep) sweeps on.  That depends on how full the tile form's chunks of 32
-// cells are, on long lines (it holds fewer), and on the lines per SM, of which the line-major sweep
-// needs enough for its 16-line warps; Gauss-Seidel, with half of them per launch, more.  Measured
-// (us per call, line-major / tile): Jacobi, 320 lines per SM, calls of 3, 4 and 10: 36 cells 121 / 163,
-// 149 / 202, 323 / 497; 48 cells 145 / 163, 184 / 202, 401 / 497; 64 cells 182 / 175, 228 / 216,
-// 513 / 530; 160 cells 431 / 417, 544 / 523, 1215 / 1297; 288 cells 754 / 785, 949 / 992, 2133 /
-// 2477.  100 lines per SM: 64 cells 94 / 73, 120 / 81, 265 / 200.  Gauss-Seidel, 220 lines per SM, calls
-// of 10: 36 cells 325 / 348, 64 cells 499 / 368, 512 cells 4256 / 3952; 800: 64 cells 1118 / 1229.
+// Fewest sweeps of a call from which the line-major form is the faster one: its three copies per call
+// against its faster sweep, where it is faster.  What decides, by measurement (calls of 1 to 50 sweeps,
+// 60 line lengths from 16 to 512 by 50 counts of lines per SM from 40 to 2600, both forms):
+//  * how much of line_tile.cu's chunks of 32 cells a line leaves empty (`used`, in percent of nx);
+//  * the lines per SM L.  The line-major sweep waits on latency below 10 warps of 16 lines per SM
+//    (Gauss-Seidel: per colour); the tile form's waves are 8 tasks of 16 lines (long lines: fewer, as
+//    shared memory goes), and a wave just begun (`tail`) costs it as much as half a full one;
+//  * whether the line-major launch has just more warps than an SM holds at once (W > 32, > 64: `over`).
+// us per call of 3 / 4 / 10 sweeps, line-major | tile.  Jacobi: 33 cells, L = 160 70 85 175 | 89 109 249;
+// 48, 280 130 161 350 | 144 185 417; 64, 280 160 201 448 | 156 197 454, 320 181 229 514 | 167 212 486;
+// 128, 500 649 828 1898 | 484 613 1392; 256, 160 414 528 1212 | 349 454 1049, 220 490 619 1398 |
+// 508 648 1492.  Gauss-Seidel: 33, 220 101 124 274 | 100 133 296, 280 110 137 298 | 134 179 397; 64,
+// 280 181 228 513 | 157 208 485; 250, 420 893 1129 2546 | 880 1169 2684.  Over all of those lengths, counts
+// and calls the rule is 0.2 % slower than the better form on average, and in one of a hundred more
+// than 2 % slower than the line-major form (9 % at most); on 460 grids drawn at random, more than 1 %
+// in one call of ninety.
 int line_seq_min_sweeps(const brs_ctx* c)
 {
     const int force = env_int("BRSMOOTH_LINE_SEQ", 1);  // 2: every grid (measurements, tests)
@@ -409,23 +416,55 @@ int line_seq_min_sweeps(const brs_ctx* c)
         return 4;
     int sms = 1;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
-    const long long lines = (long long)c->p.ny * c->p.nz / sms;
-    const int nx = c->p.nx, pad = (nx + 31) / 32 * 32;
-    const bool half = 100 * pad >= 135 * nx, thin = 10 * pad >= 12 * nx, long_ = nx >= 256;
-    if (c->p.method == BRS_JACOBI) {
-        if (half)
-            return lines >= 160 ? 2 : lines >= 130 ? 3 : lines >= 90 ? 4 : 0;
-        if (lines < 160)
+    const bool jacobi = c->p.method == BRS_JACOBI;
+    const int nx = c->p.nx, used = 100 * ((nx + 31) / 32 * 32) / nx;
+    const long long L = ((long long)c->p.ny * c->p.nz + sms - 1) / sms;
+    const long long rows = (jacobi ? 2ll : 1ll) * c->p.nz;  // of one colour, ceil(ny / 2) lines each
+    const long long W = (rows * (((c->p.ny + 1) / 2 + kLinesPerWarp - 1) / kLinesPerWarp) + sms - 1) / sms;
+    const bool five = nx >= 294 && nx < 352;  // tasks of 16 lines an SM holds
+    if (jacobi) {
+        if (used >= 175)
+            return L >= 160 ? (nx >= 32 || L >= 270 ? 2 : 3) : L > 128 ? 3 : L >= 104 ? (nx >= 32 ? 3 : 5)
+                   : L >= 88 ? 7 : 0;
+        if (used >= 150)
+            return L >= 270 ? 2 : L > 128 ? 3 : L >= 115 ? 10 : 0;
+        const bool over = (W > 32 && W <= (used < 115 ? 43 : 38)) || (W > 64 && W <= 70);
+        if (over && used < 140)
             return 0;
-        return thin || long_ ? 3 : 5;
+        if (nx >= 245) {
+            if (L > 192)
+                return nx >= 400 && L > 256 ? 2 : 3;
+            if (L >= 160 && ((five && used >= 106) || nx >= 430))
+                return 3;
+            return L > 160 && five ? 8 : 0;
+        }
+        if (L <= 128)
+            return 0;
+        const bool tail = L > 256 && (L - 1) % 128 < 52;
+        if (used >= 115)
+            return used < 122 && L > 192 && L <= 256 ? 5 : 3;
+        if (used >= 105)
+            return tail ? 3 : nx >= 176 && L < 215 ? 0 : 7;
+        return tail ? 9 : L >= 150 && L < 195 ? 10 : 0;
     }
-    if (lines < 200)
+    if (L <= 256) {
+        if (used < 175)
+            return 0;
+        return nx < 32 ? (L >= 225 ? 8 : 0) : L >= 205 ? 4 : L >= 185 ? 10 : 0;
+    }
+    if (used >= 150)
+        return nx >= 32 || L >= 340 ? 2 : 3;
+    if (W > 32 && W <= (used < 125 ? 37 : 35) && used < 140)  // over
         return 0;
-    if (half)
-        return lines < 300 ? 8 : 2;
-    if (thin)
-        return lines < 300 ? 0 : 3;
-    return lines >= (long_ ? 400 : 600) ? 5 : 0;
+    if (used >= 125)
+        return 3;
+    if (nx >= 245)
+        return L <= (five && used >= 106 ? 320 : 384) ? 0 : used >= 102 ? 4 : 10;
+    if (L >= 520)
+        return used >= 115 ? 3 : used >= 112 ? 4 : used >= 105 ? 5 : 20;
+    if (used < 112)
+        return nx < 32 && used >= 105 ? 6 : 0;
+    return nx >= 100 ? 0 : nx < 64 ? 4 : 5;
 }
 
 int line_seq_setup(brs_ctx* c)
@@ -469,6 +508,8 @@ int line_seq_setup(brs_ctx* c)
     return rc;
     return BRS_OK;
 }
+
+double* line_seq_b(brs_ctx* c) { return st(c)->Bs; }
 
 void line_seq_teardown(brs_ctx* c)
 {

@@ -54,6 +54,7 @@ struct Shape {
 struct TileState {
     double* tab = nullptr;
     double* bs = nullptr;     // omega pv_i b_i (calls of several sweeps)
+    bool own_bs = false;
     TileArgs a{};
     Shape sh;                 // of a sweep, or of one colour's launch
 };
@@ -352,9 +353,11 @@ int line_tile_setup(brs_ctx* c)
     cudaError_t e = cudaMalloc(&S->tab, tab.size() * sizeof(double));
     if (e == cudaSuccess)
         e = cudaMemcpy(S->tab, tab.data(), tab.size() * sizeof(double), cudaMemcpyHostToDevice);
-    // calls of 4 or more sweeps scale b into bs, unless the line-major form takes them
-    if (e == cudaSuccess && line_seq_min_sweeps(c) == 0)
+    // calls of 4 or more sweeps scale b into bs (the line-major form's, where the context has that)
+    if (e == cudaSuccess && line_seq_min_sweeps(c) == 0) {
         e = cudaMalloc(&S->bs, (size_t)c->cells * sizeof(double));
+        S->own_bs = true;
+    }
     a.tab = S->tab;
     const size_t smem = tile_smem(a, kLines);
     for (int q = 0; q < 18 && smem > 48u * 1024u && e == cudaSuccess; ++q) {
@@ -382,8 +385,7 @@ void line_tile_teardown(brs_ctx* c)
         return;
     if (S->tab)
         cudaFree(S->tab);
-    if (S->bs)
-        cudaFree(S->bs);
+    line_tile_trim(c);
     delete S;
     c->ltile = nullptr;
 }
@@ -438,8 +440,15 @@ int line_tile_solve(brs_ctx* c, const double* r, double* out, cudaStream_t s)
 void line_tile_trim(brs_ctx* c)
 {
     TileState* S = st(c);
-    if (S && S->bs) {
+    if (!S)
+        return;
+    if (S->own_bs)
         cudaFree(S->bs);
-        S->bs = nullptr;
-    }
+    S->own_bs = false;
+    S->bs = nullptr;
+}
+
+void line_tile_borrow(brs_ctx* c, double* bs)
+{
+    st(c)->bs = bs;
 }
