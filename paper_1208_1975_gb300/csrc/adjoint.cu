@@ -462,10 +462,27 @@ struct AdjState {
     int nblocks = 0;
     brs_ctx* xctx = nullptr;  // x-line Jacobi with omega = 1: x = M^{-1}(b + N u) in one pass
     int* xstatus = nullptr;   // xctx's own status word (its kernels report to the owner's)
+    bool tile = false;        // FP64: the block solves by the elimination from both ends
 };
 
-// FP64: both block solves on the elimination from both ends (line_tile.cu), the update in one pass
-// with its reduction.
+// Which solves an FP64 step takes.  The elimination from both ends (line_tile.cu) is a serial chain
+// of half a line, 32 lines at a time; the scan by lanes (line.cu, line_minv_kernel) does more
+// operations in log steps.  So the chain loses on long lines while an SM has few of them: time of a
+// step with the chain's over one with the scan's, by lines per SM:
+//   cells    10    18    22    26    40    48
+//    32    0.82  1.00  0.86  0.88  0.88  0.84    (10: 20.4 us / 24.8)
+//    64    1.11  1.17  0.94  0.98  0.93  0.84    (18: 41.8 / 35.6)
+//   128    1.16  1.34  1.04  0.96  1.02  0.88
+//   256    1.55  1.46  1.12  1.06  1.11  0.95
+//   512    1.34  1.50  1.12  1.05  1.00  0.90
+// From 33 cells on the sides cross at 20 lines, from 65 on at 22, from 256 on past 40.
+bool tile_solves(const brs_params& p, int sms)
+{
+    const long long per_sm = ((long long)p.ny * p.nz + sms - 1) / sms;
+    return per_sm >= (p.nx <= 32 ? 1 : p.nx <= 64 ? 20 : p.nx < 256 ? 22 : 41);
+}
+
+// FP64: both block solves, then the update in one pass with its reduction.
 int adjoint_run_f64(brs_ctx* c, double* lam, const double* u, const double* b, double* gb,
                     double* ga, cudaStream_t s)
 {
@@ -474,7 +491,7 @@ int adjoint_run_f64(brs_ctx* c, double* lam, const double* u, const double* b, d
     double* x = static_cast<double*>(c->scratch);
     double* mu = static_cast<double*>(A->mu);
     int rc;
-    if (A->xctx->ltile) {
+    if (A->tile) {
         rc = line_tile_undamped(A->xctx, u, x, b, s);
         if (rc == BRS_OK)
             rc = line_tile_solve(A->xctx, lam, mu, s);
@@ -488,9 +505,9 @@ int adjoint_run_f64(brs_ctx* c, double* lam, const double* u, const double* b, d
     // planes per item: the fewest plane steps (one more per item for its first loads) over whole
     // rounds of the resident warps
     const long long cols = (long long)p.ny * ((p.nx + 31) / 32), warps = A->nblocks * (kThreads / 32ll);
-    int kc = 4;
+    int kc = 1;
     long long best = -1;
-    for (int q = 4; q <= 32; ++q) {
+    for (int q = 1; q <= 32; ++q) {
         const long long rounds = (cols * ((p.nz + q - 1) / q) + warps - 1) / warps;
         if (best < 0 || rounds * (q + 1) < best) {
             best = rounds * (q + 1);
@@ -599,6 +616,7 @@ extern "C" int brsmooth_adjoint_sweep(brs_ctx* c, void* lam, const void* u_k, co
         A->xctx->scratch = nullptr;
         line_seq_teardown(A->xctx);
         line_tile_trim(A->xctx);
+        A->tile = A->xctx->ltile && tile_solves(c->p, sms);
         A->xstatus = A->xctx->dev_status;
         A->xctx->dev_status = c->dev_status;
     }
