@@ -4,7 +4,8 @@
 
 // Shortest rows taken: below, the digits' passes cost more than the products they replace (FP32,
 // one sweep per call: 64x61x50 36 us against 32 for two sweeps of FP32 products, 100x90x80 51
-// against 71).  Longest: 511, without 503 (the digits' sums, dst_slices.cu).
+// against 71; from 96 on FP32 contexts choose by their grid, digits_rule in plane.cu).  Longest: 511,
+// without 503 (the digits' sums, dst_slices.cu).
 constexpr int dst_slices_min(int element_size) { return element_size == 8 ? 48 : 96; }
 
 template <typename T>

@@ -111,7 +111,43 @@ struct PlaneState {
     // FP32 contexts on CUDA cores
     DstSlices<double>* slices = nullptr;
     DstSlices<float>* slices32 = nullptr;
+    bool digits_sweep = false;  // FP32: the per-sweep form by digits
+    bool digits_modes = false;  // and the calls in the x-sine basis
 };
+
+// Which FP32 transforms run by digits (the others by products of FP32 multiply-adds).  Digits cost
+// two launches more per transform and work padded to 64 x 32 modes and 128 rows, and rows off a
+// 16-byte boundary are stored one by one; past one block of rows (128 per SM) their launches come
+// again per block.  The products' work grows with n^2 and is padded to 64 cells along y, which
+// leaves them a fifth and more idle on some planes (`padded`).  Measured, time of a call by digits
+// over one by products (n x rows of a call):
+//   one sweep, Jacobi: 96 x 256 1.23, x 400 0.87, x 16500 0.82, x 24700 1.04; 106 x 400 1.04, x 1000
+//     0.92, x 12000 1.02; 128 x 272 0.97; 129 x 1500 0.78; 150 x 150 1.01, x 256 0.87
+//   one sweep, Gauss-Seidel (half of the rows per colour): 96 x 4400 1.08, x 4800 0.70, x 32300 0.82,
+//     x 47500 1.07; 106 1.05 .. 1.5 nearly everywhere; 120 x 1500 0.99, x 2880 0.89; 129 x 3000 1.17,
+//     x 15200 1.13; 130 x 77 x 100 0.82; 150 x 3000 1.07, x 4400 0.89
+//   either, from 180 modes: 0.97 and less, from 64 rows on
+//   calls of several sweeps: 96 x 3000 1.14, x 6050 1.03, x 8000 0.82, x 24700 1.16, 100 x 130 x 256
+//     0.86; 112 x 24700 1.11; 120 x 1500 1.04, x 24700 1.01; 128 1.07 and less
+void digits_rule(const brs_params& p, int sms, bool* sweep, bool* modes)
+{
+    const bool gs = p.method == BRS_CHAOTIC_GS, aligned = p.nx % 4 == 0;
+    const long long block = 128ll * sms, rows = (long long)p.ny * p.nz;
+    const long long launch = (long long)p.ny * (gs ? (p.nz + 1) / 2 : p.nz);
+    const int tiles = (p.ny + 63) / 64 * 64;
+    const bool padded = 5 * p.ny <= 4 * tiles;
+    *modes = p.nx >= 120 || ((long long)p.nz * tiles >= 7000 && (padded || rows <= block));
+    if (p.nx >= 180)
+        *sweep = true;
+    else if (aligned)
+        *sweep = p.nx >= 120 ? launch >= (gs ? 1200 : 250)
+                             : launch >= (gs ? 2400 : 400) && (padded || launch <= block);
+    else if (gs)
+        *sweep = launch >= 1900 && (p.nx >= 144 || (p.nx >= 120 && padded));
+    else
+        *sweep = p.nx >= 128 ? launch >= 250
+                             : launch >= 1000 && launch <= (padded ? block : block / 2);
+}
 
 // Map of a grid for the gather form, encoded on first use of its address.
 const CUtensorMap* grid_map(PlaneState* P, const brs_params& p, const void* ptr)
@@ -736,7 +772,7 @@ int plane_pass(brs_ctx* c, const T* uin, T* uout, const T* b, int k0, int kstep,
         }
     }
     if constexpr (sizeof(T) == 4) {
-        if (P->slices32 && P->form == 1) {
+        if (P->digits_sweep) {
             // R^ [p][y], the y solve per x-mode, and the transform back with the update
             int rc = dst_slices_rhs<float>(P->slices32, uin, b, c->p.az, T1, nullptr, ny, nz, k0,
                                            kstep, nbatch, true, s);
@@ -923,7 +959,7 @@ int modes_forward(brs_ctx* c, const void* src, void* dst, cudaStream_t s)
     const int nx = c->p.nx, ny = c->p.ny, nz = c->p.nz;
     const long long plane = (long long)nx * ny;
     cudaError_t e;
-    if (P->slices32)
+    if (P->digits_modes)
         return dst_slices_to_modes(P->slices32, static_cast<const float*>(src),
                                    static_cast<float*>(dst), ny, nz, s);
     if (modes_simt(c, P)) {
@@ -966,7 +1002,7 @@ int modes_inverse(brs_ctx* c, const void* src, void* dst, cudaStream_t s)
     const long long plane = (long long)nx * ny;
     const dim3 tgrid((unsigned)(((ny + 31) / 32) * ((nx + 31) / 32)), (unsigned)(nz < 65535 ? nz : 65535));
     cudaError_t e;
-    if (P->slices32)
+    if (P->digits_modes)
         return dst_slices_from_modes(P->slices32, static_cast<const float*>(src),
                                      static_cast<float*>(dst), ny, nz, s);
     if (modes_simt(c, P)) {
@@ -1471,7 +1507,7 @@ int modes_setup(brs_ctx* c)
     if (e == cudaSuccess)
         e = cudaMemcpy(P->mtab, all.data(), all.size() * sizeof(T), cudaMemcpyHostToDevice);
     const size_t bytes = (size_t)c->cells * sizeof(T);
-    if (P->slices32 && P->mres.C) {
+    if (P->digits_modes && P->mres.C) {
         // neither the digits' transforms nor the sweeps on chip use the per-sweep intermediates
         P->mb = P->t1;
         P->mu = P->t2;
@@ -1574,9 +1610,17 @@ int plane_setup(brs_ctx* c)
     // FP32 on CUDA cores: the transforms by digits on the tensor cores, exact to FP32's rounding
     // (BRSMOOTH_MODE_SLICES=0: products of FP32 multiply-adds)
     const char* senv = std::getenv("BRSMOOTH_MODE_SLICES");
-    if (p.dtype == BRS_F32 && P->form == 1 && !(senv && *senv && std::atoi(senv) == 0))
-        rc = dst_slices_create(p.nx, (long long)p.ny * p.nz, c->device, c->dev_status, &P->slices32);
-    if (rc == BRS_OK && !P->slices32)
+    if (p.dtype == BRS_F32 && P->form == 1 && !(senv && *senv && std::atoi(senv) == 0)) {
+        int sms = 0;
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
+        digits_rule(p, sms, &P->digits_sweep, &P->digits_modes);
+        if (P->digits_sweep || P->digits_modes)
+            rc = dst_slices_create(p.nx, (long long)p.ny * p.nz, c->device, c->dev_status,
+                                   &P->slices32);
+        if (!P->slices32)
+            P->digits_sweep = P->digits_modes = false;
+    }
+    if (rc == BRS_OK && !(P->digits_sweep && P->digits_modes))
         rc = up(&P->sx, sx);
     if (rc == BRS_OK && P->form == 2) {
         rc = up(&P->sy, sy);

@@ -1,0 +1,67 @@
+"""FP32 planes on CUDA cores: grids whose one-sweep calls and calls of several take their transforms
+from different forms (digits, products), against products alone; and no slower than those where the
+digits' passes do not pay."""
+import numpy as np
+import pytest
+
+from brs_inputs import initial_guess, rhs
+from gpu_common import TOL, rounded, to_dev, to_np
+from test_gpu_box import brs  # noqa: F401
+
+pytestmark = pytest.mark.gpu
+A = (1.0, 0.5, 0.25)
+
+
+# by turns: one-sweep calls only by digits, calls of several only, neither, both; one and two blocks of rows
+@pytest.mark.parametrize("nsweeps", [1, 3])
+@pytest.mark.parametrize("method", ["jacobi", "gs"])
+@pytest.mark.parametrize("shape", [(100, 50, 10), (96, 130, 40), (118, 64, 120), (119, 33, 7), (120, 20, 10),
+                                   (150, 30, 40), (180, 5, 3), (100, 200, 150)],
+                         ids=lambda s: "x".join(map(str, s)))
+def test_equals_products(brs, shape, method, nsweeps, monkeypatch):  # noqa: F811
+    """Each form is within the per-sweep tolerance of the exact sweep."""
+    nx, ny, nz = shape
+    u = rounded(initial_guess((nz, ny, nx)), "f32")
+    b = rounded(rhs((nz, ny, nx)), "f32")
+
+    def run():
+        with brs.Context(nx, ny, nz, A, block="plane", method=method, dtype="f32", plane_math="simt") as ctx:
+            ut, bt = to_dev(u, "f32"), to_dev(b, "f32")
+            ctx.sweep(ut, bt, nsweeps)
+            assert ctx.last_error() == 0
+            return to_np(ut)
+
+    got = run()
+    monkeypatch.setenv("BRSMOOTH_MODE_SLICES", "0")
+    assert np.max(np.abs(got - run())) <= 2 * nsweeps * TOL["f32"] * np.max(np.abs(u))
+
+
+def time(lib, n, method, sweeps):
+    """Best time of a call, in us (20 times 6 calls)."""
+    import torch
+
+    u = torch.rand(n[0] * n[1] * n[2], dtype=torch.float32, device="cuda")
+    b = torch.rand_like(u)
+    best = float("inf")
+    with lib.Context(*n, A, block="plane", method=method, dtype="f32", plane_math="simt") as ctx:
+        for k in range(25):
+            e0, e1 = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+            e0.record()
+            for _ in range(6):
+                ctx.sweep(u, b, sweeps)
+            e1.record()
+            torch.cuda.synchronize()
+            if k >= 5:
+                best = min(best, e0.elapsed_time(e1) / 6 * 1e3)
+    return best
+
+
+@pytest.mark.parametrize("n,method,sweeps", [((106, 16, 32), "gs", 1), ((106, 190, 250), "gs", 1),
+                                             ((129, 50, 60), "gs", 1), ((106, 190, 250), "jacobi", 1),
+                                             ((96, 17, 32), "gs", 3), ((96, 190, 250), "jacobi", 3)],
+                         ids=lambda v: "x".join(map(str, v)) if isinstance(v, tuple) else str(v))
+def test_no_slower_than_products(brs, n, method, sweeps, monkeypatch):  # noqa: F811
+    """By digits these took 1.16 to 1.49 times as long; 8 % for the scatter of single calls."""
+    here = time(brs, n, method, sweeps)
+    monkeypatch.setenv("BRSMOOTH_MODE_SLICES", "0")
+    assert here <= 1.08 * time(brs, n, method, sweeps)
