@@ -486,8 +486,8 @@ int brsmooth_last_error(brs_ctx* c)
     return rc;
 }
 
-int brsmooth_create_batched(int npatch, const int* dims, const brs_params* common,
-                            brs_ctx** out)
+static int create_batched(int npatch, const int* dims, const brs_params* common, bool level,
+                          brs_ctx** out)
 {
     if (!out)
         return BRS_ERR_ARG;
@@ -526,13 +526,19 @@ int brsmooth_create_batched(int npatch, const int* dims, const brs_params* commo
         return brs_cuda_status(e);
     }
     *c->dev_status = 0;
-    rc = batched_setup(c, npatch, dims);
+    rc = batched_setup(c, npatch, dims, level);
     if (rc != BRS_OK) {
         free_ctx(c);
         return rc;
     }
     *out = c;
     return BRS_OK;
+}
+
+int brsmooth_create_batched(int npatch, const int* dims, const brs_params* common,
+                            brs_ctx** out)
+{
+    return create_batched(npatch, dims, common, false, out);
 }
 
 int brsmooth_create_level(int npatch, const int* dims, const int* nbr,
@@ -563,7 +569,7 @@ int brsmooth_create_level(int npatch, const int* dims, const int* nbr,
         }
     }
     brs_ctx* c = nullptr;
-    int rc = brsmooth_create_batched(npatch, dims, common, &c);
+    int rc = create_batched(npatch, dims, common, true, &c);
     if (rc != BRS_OK)
         return rc;
     rc = level_setup(c, nbr);

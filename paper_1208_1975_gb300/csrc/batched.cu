@@ -911,16 +911,20 @@ void set_shape(brs_ctx* c, int warps, int ctas_per_sm)
 // Autotuner: time each candidate (z-chunk, warps per CTA, CTAs per SM) on scratch
 // arrays of the real patch set and keep the fastest.  Results are cached per process, keyed by
 // all that decides which candidates there are and how fast they run: the device, the patch set,
-// dtype, method, the kernel and its ring, and a chunk length fixed by BRSMOOTH_BATCH_KC.
+// dtype, method, the kernel and its ring, and a chunk length fixed by BRSMOOTH_BATCH_KC.  The cp.async
+// kernel of a level is timed itself: the plain kernel's shapes cut to the 16 warps per SM that its
+// registers allow took nine 48x43x48 patches 187 us for 20 steps (8 warps, chunks of 8) against 178
+// before and 155 now, two of 72^3 214 against 201 and 187.  The arrays are zero, so its ghosts stay so.
 struct TuneKey {
     std::vector<int> dims;
     int device, dtype, method;
+    bool level;  // a level's cp.async kernel
     int stages;  // cp.async ring slots; 0: direct loads
     int kc;      // fixed z-chunk; 0: any
     bool operator<(const TuneKey& o) const
     {
-        return std::tie(device, dtype, method, stages, kc, dims) <
-               std::tie(o.device, o.dtype, o.method, o.stages, o.kc, o.dims);
+        return std::tie(device, dtype, method, level, stages, kc, dims) <
+               std::tie(o.device, o.dtype, o.method, o.level, o.stages, o.kc, o.dims);
     }
 };
 struct TuneVal {
@@ -933,7 +937,8 @@ int autotune(brs_ctx* c)
 {
     BatchState* B = bs(c);
     const int fixed_kc = fixed_chunk();
-    TuneKey key{B->dims, c->device, c->p.dtype, c->p.method, B->async ? B->stages : 0, fixed_kc};
+    const bool level = B->async && B->level;
+    TuneKey key{B->dims, c->device, c->p.dtype, c->p.method, level, B->async ? B->stages : 0, fixed_kc};
     {
         std::lock_guard<std::mutex> lk(g_tune_mutex);
         auto it = g_tune_cache.find(key);
@@ -948,9 +953,10 @@ int autotune(brs_ctx* c)
             for (int cps : {2, 4, 5, 8}) {
                 if (w * cps > 64 || (!B->async && cps == 5))
                     continue;
-                // cp.async kernel: 8 or 20 warps per SM in CTAs of 4 warps, 16 in CTAs of 8
-                if (B->async && (w * 32 > kAsyncThreads || cps == 4 ||
-                                 !async_fits(B, w, cps, false)))
+                // cp.async kernel: 8 or 20 warps per SM in CTAs of 4 warps, 16 in CTAs of 8; a level: 8
+                // or 16 in CTAs of 4, 16 in CTAs of 8
+                if (B->async && (w * 32 > kAsyncThreads || cps == (level ? 5 : 4) ||
+                                 (level && w * cps > 16) || !async_fits(B, w, cps, level)))
                     continue;
                 cands.push_back({kc, w, cps});
             }
@@ -1020,7 +1026,7 @@ int autotune(brs_ctx* c)
 
 }  // namespace
 
-int batched_setup(brs_ctx* c, int npatch, const int* dims)
+int batched_setup(brs_ctx* c, int npatch, const int* dims, bool level)
 {
     BatchState* B = new BatchState();
     c->batch = B;
@@ -1100,18 +1106,13 @@ int batched_setup(brs_ctx* c, int npatch, const int* dims)
         set_shape(c, 8, B->async ? 2 : 4);
         return build_items(c, kc ? kc : 8);
     }
-    return autotune(c);
+    return level && B->async ? BRS_OK : autotune(c);
 }
 
 int level_setup(brs_ctx* c, const int* nbr)
 {
     BatchState* B = bs(c);
     B->level = true;
-    // a level's rings also hold its x ghosts, and its kernel has more registers
-    while (B->async && B->ctas_per_sm > 1 &&
-           (B->warps * B->ctas_per_sm > 16 ||
-            !async_fits(B, B->warps, B->ctas_per_sm, true)))
-        set_shape(c, B->warps, B->ctas_per_sm - 1);
     // boundary-cell chunks per patch (every dim >= 2, checked by the caller)
     std::vector<int> chunk_patch;
     long long gtotal = 0;
@@ -1127,8 +1128,15 @@ int level_setup(brs_ctx* c, const int* nbr)
             chunk_patch.push_back(q);
     }
     B->nchunks = (int)chunk_patch.size();
-    cudaError_t e = cudaMemcpy(B->d_desc, B->h_desc.data(), sizeof(PatchDesc) * B->npatch,
-                               cudaMemcpyHostToDevice);
+    const bool tuned = B->d_desc;  // direct loads, or BRSMOOTH_BATCH_NOTUNE
+    // a level's rings also hold its x ghosts
+    while (tuned && B->async && B->ctas_per_sm > 1 &&
+           !async_fits(B, B->warps, B->ctas_per_sm, true))
+        set_shape(c, B->warps, B->ctas_per_sm - 1);
+    cudaError_t e = cudaSuccess;
+    if (tuned)
+        e = cudaMemcpy(B->d_desc, B->h_desc.data(), sizeof(PatchDesc) * B->npatch,
+                       cudaMemcpyHostToDevice);
     if (e == cudaSuccess)
         e = cudaMalloc(&B->d_chunk_patch, sizeof(int) * chunk_patch.size());
     if (e == cudaSuccess)
@@ -1171,7 +1179,7 @@ int level_setup(brs_ctx* c, const int* nbr)
             e = cudaMemcpy(B->d_push, push.data(), sizeof(long long) * push.size(),
                            cudaMemcpyHostToDevice);
     }
-    return brs_cuda_status(e);
+    return e != cudaSuccess || tuned ? brs_cuda_status(e) : autotune(c);
 }
 
 void batched_teardown(brs_ctx* c)

@@ -2,7 +2,8 @@
 #pragma once
 #include "brs_internal.cuh"
 
-int batched_setup(brs_ctx* c, int npatch, const int* dims);
+// level: level_setup follows (it finds the launch shape with the level's own kernel).
+int batched_setup(brs_ctx* c, int npatch, const int* dims, bool level);
 // Turns a batched context into a level: face-neighbour table (6 per patch, validated by
 // the caller), boundary-cell chunks and the b_eff array.
 int level_setup(brs_ctx* c, const int* nbr);
