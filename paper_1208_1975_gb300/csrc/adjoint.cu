@@ -467,19 +467,25 @@ struct AdjState {
 
 // Which solves an FP64 step takes.  The elimination from both ends (line_tile.cu) is a serial chain
 // of half a line, 32 lines at a time; the scan by lanes (line.cu, line_minv_kernel) does more
-// operations in log steps.  So the chain loses on long lines while an SM has few of them: time of a
-// step with the chain's over one with the scan's, by lines per SM:
-//   cells    10    18    22    26    40    48
-//    32    0.82  1.00  0.86  0.88  0.88  0.84    (10: 20.4 us / 24.8)
-//    64    1.11  1.17  0.94  0.98  0.93  0.84    (18: 41.8 / 35.6)
-//   128    1.16  1.34  1.04  0.96  1.02  0.88
-//   256    1.55  1.46  1.12  1.06  1.11  0.95
-//   512    1.34  1.50  1.12  1.05  1.00  0.90
-// From 33 cells on the sides cross at 20 lines, from 65 on at 22, from 256 on past 40.
+// operations in log steps.  So the chain loses on long lines while an SM has few of them, least
+// where its tiles come to whole rounds: time of a step with the chain's over one with the scan's, by
+// lines per SM:
+//   cells     8    10    12    16    18    20    22    27    40    46
+//    33    0.87  0.89  0.89  1.12  0.95  0.84  0.81  0.84  0.84  0.81
+//    57    1.01  1.03  1.04  1.26  1.13  0.97  0.92  0.97  0.95  0.89
+//    77    1.12  0.95  0.97  1.21  1.07  0.96  0.87  0.83  0.86  0.76
+//   113    1.24  1.12  1.11  1.37  1.28  1.12  1.01  0.94  1.00  0.88
+//   201    1.35  1.15  1.13  1.44  1.29  1.10  1.01  0.94  0.94  0.87
+//   333    1.47  1.26  1.26  1.60  1.47  1.19  1.06  1.04  1.09  0.92
+//   501    1.33  1.08  1.06  1.31  1.23  1.06  0.95  0.83  0.87  0.74
+// and with rows that the scan moves as vectors (256, 384 and 512 cells) up to 1.12 from 22 lines on,
+// 1.02 .. 1.11 at 40.
 bool tile_solves(const brs_params& p, int sms)
 {
     const long long per_sm = ((long long)p.ny * p.nz + sms - 1) / sms;
-    return per_sm >= (p.nx <= 32 ? 1 : p.nx <= 64 ? 20 : p.nx < 256 ? 22 : 41);
+    if (p.nx <= 32 || (p.nx <= 64 && per_sm <= 12) || (p.nx <= 96 && per_sm >= 9 && per_sm <= 12))
+        return true;
+    return per_sm >= (p.nx <= 64 ? 20 : p.nx >= 256 && p.nx % 128 == 0 ? 41 : 22);
 }
 
 // FP64: both block solves, then the update in one pass with its reduction.
