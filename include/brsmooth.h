@@ -130,8 +130,8 @@ typedef struct brs_params {
  * ny <= 512 transform by digits on the tensor cores, exact to the type's rounding of each row's
  * 2-norm, and hold the digits of one block of rows (at most 128 rows per SM, 14 (8) bytes per
  * cell); other rows are transformed by products in the type, and so are, in FP32, those of
- * one-sweep calls below 180 modes and of longer calls below 120 where the grid makes the
- * products the faster form.
+ * one-sweep calls below 180 modes where the grid makes the products the faster form, and of
+ * longer calls on few rows below 120.
  * FP64 contexts, and FP32 contexts where TMA can stage rows of ny elements (ny times 4 bytes a
  * multiple of 16, ny a whole number of the lane chunks of the line solve) or, on CUDA cores,
  * where nx >= 48, also hold the x-sine form of calls of several sweeps: at most two more grids

@@ -124,29 +124,38 @@ struct PlaneState {
 //   one sweep, Jacobi: 96 x 256 1.23, x 400 0.87, x 16500 0.82, x 24700 1.04; 106 x 400 1.04, x 1000
 //     0.92, x 12000 1.02; 128 x 272 0.97; 129 x 1500 0.78; 150 x 150 1.01, x 256 0.87
 //   one sweep, Gauss-Seidel (half of the rows per colour): 96 x 4400 1.08, x 4800 0.70, x 32300 0.82,
-//     x 47500 1.07; 106 1.05 .. 1.5 nearly everywhere; 120 x 1500 0.99, x 2880 0.89; 129 x 3000 1.17,
-//     x 15200 1.13; 130 x 77 x 100 0.82; 150 x 3000 1.07, x 4400 0.89
+//     x 47500 1.07; 106 1.05 .. 1.5 nearly everywhere, but x 20 x 200 0.9; 120 x 1500 0.99, x 2880 0.89;
+//     127 x 5 x 200 1.16; 128 x 16 x 64 1.08, x 100 x 4 0.98; 129 x 3000 1.17, x 15200 1.13; 130 x 77 x
+//     100 0.82, x 20 x 200 0.75; 150 x 3000 1.07, x 4400 0.89
 //   either, from 180 modes: 0.97 and less, from 64 rows on
-//   calls of several sweeps: 96 x 3000 1.14, x 6050 1.03, x 8000 0.82, x 24700 1.16, 100 x 130 x 256
-//     0.86; 112 x 24700 1.11; 120 x 1500 1.04, x 24700 1.01; 128 1.07 and less
+// Calls of several sweeps, at most 1.24, are left to digits, which are the more exact form, except
+// where the call would take longer than by the products of all its transforms that came first (two
+// sweeps, by the form of then: 96 x 64 .. 1024 1.01 .. 1.13, x 2000 1.03, x 4000 0.88; 128 0.9; rows of
+// y that TMA cannot stage 0.85 and less).
 void digits_rule(const brs_params& p, int sms, bool* sweep, bool* modes)
 {
     const bool gs = p.method == BRS_CHAOTIC_GS, aligned = p.nx % 4 == 0;
-    const long long block = 128ll * sms, rows = (long long)p.ny * p.nz;
-    const long long launch = (long long)p.ny * (gs ? (p.nz + 1) / 2 : p.nz);
-    const int tiles = (p.ny + 63) / 64 * 64;
+    const int planes = gs ? (p.nz + 1) / 2 : p.nz, tiles = (p.ny + 63) / 64 * 64;
+    const long long block = 128ll * sms, launch = (long long)p.ny * planes;
+    const long long padded_rows = (long long)tiles * planes;
     const bool padded = 5 * p.ny <= 4 * tiles;
-    *modes = p.nx >= 120 || ((long long)p.nz * tiles >= 7000 && (padded || rows <= block));
+    *modes = p.nx >= 120 || p.ny % 4 != 0 || (long long)p.ny * p.nz >= 3000 ||
+             (long long)tiles * p.nz >= 4500;
     if (p.nx >= 180)
         *sweep = true;
+    else if (!gs)
+        *sweep = p.nx >= (aligned ? 120 : 128)
+                     ? launch >= 250
+                     : launch >= (aligned ? 400 : 600) &&
+                           (aligned && padded || launch <= (aligned || padded ? block : block / 2));
+    else if (p.nx >= (aligned ? 120 : 144))
+        *sweep = launch >= (aligned ? 1200 : 1900) || padded_rows >= 4800 || (aligned && p.ny >= 50);
     else if (aligned)
-        *sweep = p.nx >= 120 ? launch >= (gs ? 1200 : 250)
-                             : launch >= (gs ? 2400 : 400) && (padded || launch <= block);
-    else if (gs)
-        *sweep = launch >= 1900 && (p.nx >= 144 || (p.nx >= 120 && padded));
+        *sweep = (launch >= 2450 || padded_rows >= 6000) && (padded || launch <= block);
+    else if (p.nx >= 120)
+        *sweep = padded && (launch >= 1900 || (p.nx > 128 && padded_rows >= 4800));
     else
-        *sweep = p.nx >= 128 ? launch >= 250
-                             : launch >= 1000 && launch <= (padded ? block : block / 2);
+        *sweep = padded && padded_rows >= 8000 && launch <= block / 2;
 }
 
 // Map of a grid for the gather form, encoded on first use of its address.

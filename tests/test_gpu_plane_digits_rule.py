@@ -58,10 +58,11 @@ def time(lib, n, method, sweeps):
 
 @pytest.mark.parametrize("n,method,sweeps", [((106, 16, 32), "gs", 1), ((106, 190, 250), "gs", 1),
                                              ((129, 50, 60), "gs", 1), ((106, 190, 250), "jacobi", 1),
-                                             ((96, 17, 32), "gs", 3), ((96, 190, 250), "jacobi", 3)],
+                                             ((96, 16, 32), "gs", 2), ((106, 16, 64), "jacobi", 2)],
                          ids=lambda v: "x".join(map(str, v)) if isinstance(v, tuple) else str(v))
 def test_no_slower_than_products(brs, n, method, sweeps, monkeypatch):  # noqa: F811
-    """By digits these took 1.16 to 1.49 times as long; 8 % for the scatter of single calls."""
+    """By digits these took 1.16 to 1.49 times as long (the calls of two sweeps also longer than by the
+    form that came first); 8 % for the scatter of single calls."""
     here = time(brs, n, method, sweeps)
     monkeypatch.setenv("BRSMOOTH_MODE_SLICES", "0")
     assert here <= 1.08 * time(brs, n, method, sweeps)
