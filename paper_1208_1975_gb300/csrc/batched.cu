@@ -1000,8 +1000,8 @@ int autotune(brs_ctx* c)
             cudaEventElapsedTime(&t, e0, e1);
             ms = t < ms ? t : ms;
         }
-        // cp.async kernel: fewer warps where more gain nothing
-        if (rc == BRS_OK && ms < (B->async ? 0.98f : 1.0f) * best_ms) {
+        // plain cp.async kernel: fewer warps where more gain nothing
+        if (rc == BRS_OK && ms < (B->async && !level ? 0.98f : 1.0f) * best_ms) {
             best_ms = ms;
             best = v;
         }
