@@ -12,7 +12,7 @@
 // 6 x 3.75 operations per cell for the transforms and about 26 for the whole update, against 512
 // for the dense inverse (64 and the folds by parity classes): FP64 is bound by its pipe (626 G
 // operations/s, 24 Gcell/s; measured 19.5 at 256^3), FP32 by HBM (12 bytes per cell) and the
-// trips through shared memory (324 Gcell/s, 0.57 of the measured copy, Jacobi).
+// trips through shared memory (320 Gcell/s, 0.57 of the measured copy, Jacobi).
 //
 // A CTA holds NB boxes in shared memory.  Five stages, one thread per line of cells, a line in
 // registers: x rows (gather the right-hand side from global memory, transform), y lines,
